@@ -403,38 +403,50 @@ __global__ void k_collapse_leaves(Node *nodes, int n_internal, int leaf_size) {
   nodes[p].child.y = out[1];
 }
 
-// The 4-wide form the traversal reads, one thread per binary node: wide node
-// p lists binary node p's grandchildren -- a child that is a leaf stands for
-// itself -- with the boxes the binary nodes hold for them (already grown, see
-// k_lbvh_boxes), so a search from any binary node tests the same boxes as a
-// binary search would, two levels per node fetch.  Child order: left
-// subtree first.
+// The 4-wide form the traversal reads, one thread per binary node: wide node p
+// starts from binary node p's two children and opens, until it has four, the
+// inner one with the largest box (the one a ray is likeliest to enter), with
+// the boxes the binary nodes hold for them (already grown, see k_lbvh_boxes),
+// so a search from any binary node tests boxes a binary search would.  Unused
+// lanes get an inverted infinite box.
 __global__ void k_widen(const Node *nodes, int n_internal, Node4 *wide) {
   int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n_internal) return;
-  const Node b = nodes[p];
   float bx[4][6];  // lo.x, hi.x, lo.y, hi.y, lo.z, hi.z per child
   int code[4];
-  int m = 0;
-  auto put = [&](float4 xy, float z0, float z1, int c) {
+  float area[4];   // half the surface of an inner child's box; -1: a leaf or unused
+  auto put = [&](int m, float4 xy, float z0, float z1, int c) {
     bx[m][0] = xy.x; bx[m][1] = xy.y; bx[m][2] = xy.z; bx[m][3] = xy.w; bx[m][4] = z0; bx[m][5] = z1;
-    code[m++] = c;
+    code[m] = c;
+    const float dx = xy.y - xy.x, dy = xy.w - xy.z, dz = z1 - z0;
+    area[m] = c >= 0 ? dx * dy + dy * dz + dz * dx : -1.0f;
   };
 #pragma unroll
-  for (int side = 0; side < 2; side++) {
-    const int c = side == 0 ? b.child.x : b.child.y;
-    if (c < 0) {
-      if (side == 0) put(b.lxy, b.lrz.x, b.lrz.y, c);
-      else put(b.rxy, b.lrz.z, b.lrz.w, c);
-    } else {
-      const Node g = nodes[c];
-      put(g.lxy, g.lrz.x, g.lrz.y, g.child.x);
-      put(g.rxy, g.lrz.z, g.lrz.w, g.child.y);
-    }
-  }
-  for (int q = m; q < 4; q++) {
-    for (int k = 0; k < 6; k++) bx[q][k] = 0.0f;
+  for (int q = 0; q < 4; q++) {
+    bx[q][0] = bx[q][2] = bx[q][4] = kInf;
+    bx[q][1] = bx[q][3] = bx[q][5] = -kInf;
     code[q] = kNoChild;
+    area[q] = -1.0f;
+  }
+  auto open = [&](int at, int next, int node) {
+    const Node g = nodes[node];
+    // (constant indices keep the lanes in registers)
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      if (q == at) put(q, g.lxy, g.lrz.x, g.lrz.y, g.child.x);
+      if (q == next) put(q, g.rxy, g.lrz.z, g.lrz.w, g.child.y);
+    }
+  };
+  open(0, 1, p);
+#pragma unroll
+  for (int m = 2; m < 4; m++) {
+    int at = -1, node = 0;
+    float best = -1.0f;
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+      if (q < m && area[q] > best) { best = area[q]; at = q; node = code[q]; }
+    if (at < 0) break;
+    open(at, m, node);
   }
   Node4 w;
   w.lox = make_float4(bx[0][0], bx[1][0], bx[2][0], bx[3][0]);

@@ -233,60 +233,76 @@ struct WarpCount {
   }
 };
 
+// What a triangle test found: an accepted hit at distance t (t64 in FP64), or
+// (deferring variants) an ambiguous one, or nothing.
+struct TriHit {
+  float t;
+  double t64;
+  int id;
+  bool ok, amb;
+};
+
+// Test leaf slot `slot` against ray r; hits beyond `tmax` are dropped.
 template <int kP, bool kCount>
-__device__ __forceinline__ void consider_tri(const DevScene &sc, const Tri *tris, const Ray &r, const RaySrc &rs,
-                                             double dns64, Best &best, int slot, const WarpCount &n_tris, float tlim) {
+__device__ __forceinline__ TriHit test_tri(const Tri *tris, const Ray &r, const RaySrc &rs, double dns64, int slot,
+                                           const WarpCount &n_tris, float tmax) {
   constexpr bool kDefer = Prec<kP>::defer, kAll64 = Prec<kP>::all64;
   if (kCount) n_tris++;
   const Tri *tp = tris + slot;
-  float4 v0 = __ldg(&tp->v0), v1 = __ldg(&tp->v1), v2 = __ldg(&tp->v2);
-  float t;
-  double t64 = 0.0;
-  bool has64 = false;
-  bool amb = false;
+  const float4 v0 = __ldg(&tp->v0), v1 = __ldg(&tp->v1), v2 = __ldg(&tp->v2);
+  TriHit h = {0.0f, 0.0, __float_as_int(v1.w), false, false};
   if (kAll64) {
     // FP64: every candidate in float64 Moller-Trumbore on the float64 ray
     double3 o, d;
     rs.get(o, d);
     double tt;
-    if (!hit_mt64(o, d, v0, v1, v2, tt)) return;
-    if (!(tt > (double)r.t_eps && (dns64 == 0.0 || tt * dns64 > (double)r.t_eps))) return;
-    t64 = tt;
-    has64 = true;
-    t = (float)tt;
-  } else {
-    t = hit_watertight(r, v0, v1, v2, amb);
+    if (!hit_mt64(o, d, v0, v1, v2, tt)) return h;
+    if (!(tt > (double)r.t_eps && (dns64 == 0.0 || tt * dns64 > (double)r.t_eps))) return h;
+    h.t64 = tt;
+    h.t = (float)tt;
+    h.ok = !(h.t > tmax);
+    return h;
   }
-  if (kAll64) {
-  } else {
-    // MIXED: an ambiguous candidate is decided in float64 after the search
-    if (kDefer && amb && pend_add(rs, slot | kPendAmb)) return;
-    if (!(t < kInf && accept_hit(r, t))) return;
-  }
-  if (t > tlim) return;  // sub-domain: beyond the tile (see k_trace_tiled)
-  int id = __float_as_int(v1.w);
+  bool amb;
+  h.t = hit_watertight(r, v0, v1, v2, amb);
+  h.ok = h.t < kInf && accept_hit(r, h.t) && !(h.t > tmax);
+  h.amb = kDefer && amb;
+  return h;
+}
+
+// The window of distances around the best hit that is settled in float64.
+__device__ __forceinline__ float tie_window(float t) { return 1e-5f * fabsf(t) + 1e-4f; }
+
+// A hit (or an ambiguous test) of leaf slot `slot` against the best hit so
+// far.
+template <int kP>
+__device__ __forceinline__ void weigh_hit(const RaySrc &rs, Best &best, int slot, const TriHit &h) {
+  constexpr bool kDefer = Prec<kP>::defer;
+  // MIXED: an ambiguous candidate is decided in float64 after the search
+  if (kDefer && h.amb && pend_add(rs, slot | kPendAmb)) return;
+  if (!h.ok) return;
   if (kP == kPF32) {
-    if (t < best.t || (t == best.t && id < best.id)) { best.t = t; best.slot = slot; best.id = id; }
+    if (h.t < best.t || (h.t == best.t && h.id < best.id)) { best.t = h.t; best.slot = slot; best.id = h.id; }
     return;
   }
   // MIXED and FP64: a clearly nearer or farther float32 distance decides; a
   // near tie is settled in float64, where distances within 1e-9 relative tie
   // and go to the lowest triangle index (MIXED: after the search)
-  float win = 1e-5f * fabsf(best.t) + 1e-4f;
-  if (best.slot < 0 || t < best.t - win) {
-    best.t = t; best.slot = slot; best.id = id; best.t64 = t64; best.has64 = has64;
+  const float win = tie_window(best.t);
+  if (best.slot < 0 || h.t < best.t - win) {
+    best.t = h.t; best.slot = slot; best.id = h.id; best.t64 = h.t64; best.has64 = !kDefer;
     return;
   }
-  if (t > best.t + win) return;
+  if (h.t > best.t + win) return;
   if (kDefer) {
-    if (!pend_add(rs, slot) && (t < best.t || (t == best.t && id < best.id))) {
-      best.t = t; best.slot = slot; best.id = id; best.t64 = 0.0; best.has64 = false;
+    if (!pend_add(rs, slot) && (h.t < best.t || (h.t == best.t && h.id < best.id))) {
+      best.t = h.t; best.slot = slot; best.id = h.id; best.t64 = 0.0; best.has64 = false;
     }
     return;
   }
-  double tol = 1e-9 * (1.0 + fabs(t64));
-  if (t64 < best.t64 - tol || (fabs(t64 - best.t64) <= tol && id < best.id)) {
-    best.t = (float)t64; best.slot = slot; best.id = id; best.t64 = t64; best.has64 = true;
+  const double tol = 1e-9 * (1.0 + fabs(h.t64));
+  if (h.t64 < best.t64 - tol || (fabs(h.t64 - best.t64) <= tol && h.id < best.id)) {
+    best.t = (float)h.t64; best.slot = slot; best.id = h.id; best.t64 = h.t64; best.has64 = true;
   }
 }
 
@@ -360,139 +376,382 @@ __device__ __forceinline__ void sort_pair(float &ka, int &ca, float &kb, int &cb
   ca = c;
 }
 
+__device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
+
+constexpr int kTraceThreads = 128;
+
+// Triangle tests a warp owes: (lane, leaf code) pairs that its lanes' node
+// steps exposed.  Once there are kPairTest of them (or the phase ends) the warp
+// tests 32 at a time, each lane one pair, whichever lane's ray it belongs to.
+// A node step exposes a triangle on about one lane in six, so testing them
+// where they arise ran the triangle code for 4.4 of 32 lanes nearly as often as
+// the node code; by pairs it runs for 18 (both counted on the CPU over the
+// axis rays of 4 district sources).  The best hits the node steps cull by are
+// then up to kPairTest tests old, which costs 2 % more node visits at 12 (8
+// and 16 measured 2-5 % slower).
+constexpr int kPairTest = 12;
+constexpr int kPairCap = 4 * 32 + kPairTest;  // a step adds at most four per lane
+template <int kWarps>
+struct PairQueue {
+  int code[kWarps][kPairCap];
+  int n[kWarps];
+  unsigned char lane[kWarps][kPairCap];
+};
+struct WarpPairs {
+  int *code, *n;
+  unsigned char *lane;
+};
+template <int kWarps>
+__device__ __forceinline__ WarpPairs warp_pairs(PairQueue<kWarps> &q) {
+  const int w = threadIdx.x >> 5;
+  if (lane_id() == 0) q.n[w] = 0;
+  __syncwarp();
+  return WarpPairs{q.code[w], &q.n[w], q.lane[w]};
+}
+
 // A closest-hit search that can stop after any node and resume later: its
-// state is the current node, the stack (an array the caller keeps) and the
-// best hit so far.
+// state is the current node, the stack (an array the caller keeps: the inner
+// children not yet visited) and the best hit so far.
 struct HitSearch {
-  int node, sp, visits;
+  int node, sp, budget;
   Best best;
-  __device__ __forceinline__ void start(int root) {
+  __device__ __forceinline__ void start(int root, int64_t n_tris) {
     node = root;
     sp = 0;
-    visits = 0;
+    budget = (int)n_tris + 64;
     best.t = kInf;
     best.slot = -1;
     best.id = 0x7fffffff;
     best.t64 = 0.0;
     best.has64 = false;
   }
-  // One wide node of the traversal (the boxes of its up to four children in
-  // one 128-byte fetch; the nearest child hit next, the others pushed
-  // farthest first) and the leaves it exposes.  False once the search is
-  // over.
-  template <int kP, bool kCount, bool kLeaves>
-  __device__ __forceinline__ bool step(const DevScene &sc, const Node4 *nodes, const Tri *tris, int64_t n_tri,
-                                       const Ray &r, const RaySrc &rs, double dns64, int *stack, int *err,
-                                       const WarpCount &n_nodes, const WarpCount &n_tris, float tlim) {
-    if (n_tri == 0 || node == kNoChild) return false;
-    // the leaves this step tests: child codes in `lc`, the lanes in `lm`
-    int4 lc = make_int4(node, 0, 0, 0);
-    unsigned lm = 0;
-    bool more = true;
-    if (node < 0) {
-      // a leaf: the root of a one-leaf hierarchy, or (kLeaves) the rest of a
-      // larger leaf put back on the stack (below)
-      lm = 1;
-      if (kLeaves && sp > 0) node = stack[--sp];
-      else more = false;
-    } else {
-      // a well-formed BVH is visited at most once per node; the bound only
-      // guarantees termination should the structure ever be malformed
-      if (++visits > (int)n_tri + 64) {
-        atomicExch(err, BT_E_TIMEOUT);
-        return false;
-      }
-      const Node4 *nd = nodes + node;
-      if (kCount) n_nodes++;
-      const float4 lox = __ldg(&nd->lox), hix = __ldg(&nd->hix), loy = __ldg(&nd->loy), hiy = __ldg(&nd->hiy);
-      const float4 loz = __ldg(&nd->loz), hiz = __ldg(&nd->hiz);
-      const int4 ch = __ldg(&nd->child);
-      // in MIXED and FP64 mode near ties must still be visited
-      const float tmax = fminf(kP != kPF32 ? best.t + (1e-5f * fabsf(best.t) + 1e-4f) : best.t, tlim);
-      const float3 oi = origin_scaled(r);
-      float k0, k1, k2, k3;
-      const bool h0 = slab(r, oi, lox.x, hix.x, loy.x, hiy.x, loz.x, hiz.x, tmax, k0) && ch.x != kNoChild;
-      const bool h1 = slab(r, oi, lox.y, hix.y, loy.y, hiy.y, loz.y, hiz.y, tmax, k1) && ch.y != kNoChild;
-      const bool h2 = slab(r, oi, lox.z, hix.z, loy.z, hiy.z, loz.z, hiz.z, tmax, k2) && ch.z != kNoChild;
-      const bool h3 = slab(r, oi, lox.w, hix.w, loy.w, hiy.w, loz.w, hiz.w, tmax, k3) && ch.w != kNoChild;
-      lc = ch;
-      lm = (unsigned)(h0 && ch.x < 0) | (unsigned)(h1 && ch.y < 0) << 1 | (unsigned)(h2 && ch.z < 0) << 2 |
-           (unsigned)(h3 && ch.w < 0) << 3;
-      // inner children hit, nearest first (a sorting network on the entry
-      // distances; misses sort last)
-      int c0 = ch.x, c1 = ch.y, c2 = ch.z, c3 = ch.w;
-      k0 = h0 && c0 >= 0 ? k0 : kInf;
-      k1 = h1 && c1 >= 0 ? k1 : kInf;
-      k2 = h2 && c2 >= 0 ? k2 : kInf;
-      k3 = h3 && c3 >= 0 ? k3 : kInf;
-      const int ni = (k0 < kInf) + (k1 < kInf) + (k2 < kInf) + (k3 < kInf);
-      sort_pair(k0, c0, k1, c1);
-      sort_pair(k2, c2, k3, c3);
-      sort_pair(k0, c0, k2, c2);
-      sort_pair(k1, c1, k3, c3);
-      sort_pair(k1, c1, k2, c2);
-      if (ni > 0) {
-        if (sp + ni - 1 <= kStackDepth) {
-          if (ni > 3) stack[sp++] = c3;
-          if (ni > 2) stack[sp++] = c2;
-          if (ni > 1) stack[sp++] = c1;
-        } else {
-          atomicExch(err, BT_E_QUEUE_FULL);
-        }
-        node = c0;
-      } else if (sp > 0) {
-        node = stack[--sp];
-      } else {
-        more = false;
+  // Distances beyond which nothing is of interest: in MIXED and FP64 mode
+  // near ties must still be visited.
+  template <int kP>
+  __device__ __forceinline__ float limit(float tlim) const {
+    return fminf(kP != kPF32 ? best.t + tie_window(best.t) : best.t, tlim);
+  }
+};
+
+// Test the warp's `n` pairs, 32 at a time.  Each lane takes one pair and makes
+// its owner's ray again from the rows in shared memory (which costs less than
+// holding the test's part of every ray in registers); the hits then go back to
+// their owners, one per owner and round, through a mailbox in the pairs' own
+// (read) entries.  Warp-collective; t_eps, dns, dns64 and tlim are the calling
+// lane's own.
+template <int kP, bool kCount, bool kLeaves>
+__device__ __forceinline__ void test_pairs(const WarpPairs &wp, int n, const Tri *tris, bool lane_tris, float t_eps,
+                                           float dns, const RaySrc &rs, double dns64, HitSearch &hs,
+                                           const WarpCount &n_tris, float tlim, int lg = 0) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = (int)lane_id();
+  volatile int *const mail = wp.code;
+  for (int base = 0; base < n; base += 32) {
+    const bool have = base + lane < n;
+    int code = 0, owner = lane;
+    if (have) {
+      code = wp.code[base + lane];
+      owner = wp.lane[base + lane];
+    }
+    __syncwarp();
+    RaySrc qs = rs;
+    const int col = (owner >> lg) - (lane >> lg);  // the owner's column, from one's own
+    const float *h6 = rs.hi + col;
+    const float3 qo = make_float3(h6[0], h6[rs.stride], h6[2 * rs.stride]);
+    const float3 qd = make_float3(h6[3 * rs.stride], h6[4 * rs.stride], h6[5 * rs.stride]);
+    const Ray q = make_ray(qo, qd, lane_tris ? __shfl_sync(kAll, t_eps, owner) : t_eps,
+                           kP == kPF64 ? 0.0f : __shfl_sync(kAll, dns, owner));
+    const Tri *qt = tris;
+    if (lane_tris) qt = (const Tri *)__shfl_sync(kAll, (unsigned long long)tris, owner);
+    double qdns64 = 0.0;
+    if (kP == kPF64) {
+      qdns64 = __shfl_sync(kAll, dns64, owner);
+      qs.dv += col;
+    }
+    int left = 1;
+    if (kLeaves) {
+      left = have ? leaf_count(code) : 0;
+      code = leaf_slot(code);
+    }
+    // (kLeaves: a pair may stand for several consecutive triangles)
+    for (int j = 0; kLeaves ? __any_sync(kAll, j < left) != 0 : j < 1; j++) {
+      const float tmax = __shfl_sync(kAll, hs.limit<kP>(tlim), owner);
+      TriHit h = {0.0f, 0.0, 0, false, false};
+      if (kLeaves ? j < left : have) h = test_tri<kP, kCount>(qt, q, qs, qdns64, code + j, n_tris, tmax);
+      bool todo = h.ok || h.amb;
+      while (__any_sync(kAll, todo)) {
+        mail[lane] = -1;
+        __syncwarp();
+        if (todo) mail[owner] = lane;
+        __syncwarp();
+        const int from = mail[lane];
+        if (todo && mail[owner] == lane) todo = false;
+        const int src = from < 0 ? lane : from;
+        TriHit g;
+        g.t = __shfl_sync(kAll, h.t, src);
+        g.id = __shfl_sync(kAll, h.id, src);
+        g.t64 = kP == kPF64 ? __shfl_sync(kAll, h.t64, src) : 0.0;
+        const int flags = __shfl_sync(kAll, (int)h.ok | (int)h.amb << 1, src);
+        const int slot = __shfl_sync(kAll, code + j, src);
+        g.ok = flags & 1;
+        g.amb = flags >> 1;
+        if (from >= 0) weigh_hit<kP>(rs, hs.best, slot, g);
+        __syncwarp();
       }
     }
+  }
+  if (lane == 0) *wp.n = 0;
+  __syncwarp();
+}
+
+// The search phase of a warp: every lane with `more` nodes to visit takes node
+// steps until at most `few` lanes have nodes left.  kPairs: the exposed
+// triangles are tested by pairs, else each lane tests its own at once.
+// lane_tris: the lanes' scenes differ.  Warp-collective.
+//
+// A node step is one wide node: the boxes of its up to four children in one
+// 128-byte fetch, each axis' near and far planes told apart by the sign of the
+// ray's direction; the nearest inner child hit next, the others pushed
+// farthest first.
+template <int kP, bool kCount, bool kLeaves, bool kPairs>
+__device__ __forceinline__ void search_phase(const DevScene &sc, bool lane_tris, const Ray &r, const RaySrc &rs,
+                                             double dns64, int *stack, int *err, HitSearch &hs, bool &more,
+                                             const WarpPairs &wp, const WarpCount &n_nodes, const WarpCount &n_tris,
+                                             float tlim, int few) {
+  // the hot fields in registers: in a batch `sc` lives in device memory and
+  // would otherwise be re-read on every node
+  const char *const nodes = (const char *)sc.nodes;
+  const Tri *const tris = sc.tris;
+  const float3 inv = r.inv, oi = origin_scaled(r);
+  const float t_eps = r.t_eps, dns = r.dns;
+  auto expose = [&](int c, int pos) {
+    wp.code[pos] = ~c;
+    wp.lane[pos] = (unsigned char)lane_id();
+  };
+  // the leaves ~lc of the lanes in lm, tested at once (a leaf of several
+  // triangles is one run of slots)
+  auto test_now = [&](int4 lc, unsigned lm) {
 #pragma unroll 1
     while (lm) {
       const int c = __ffs(lm) - 1;
       lm &= lm - 1;
       const int v = ~(c == 0 ? lc.x : c == 1 ? lc.y : c == 2 ? lc.z : lc.w);
-      if (kLeaves && (v >> kLeafShift)) {
-        // a leaf of several triangles: its first now, the rest as a leaf of
-        // one triangle fewer at a later step, so that a step still tests at
-        // most one triangle per leaf
-        const int rest = ~((leaf_slot(v) + 1) | (((v >> kLeafShift) - 1) << kLeafShift));
-        if (!more) {
-          node = rest;
-          more = true;
-        } else if (sp < kStackDepth) {
-          stack[sp++] = rest;
-        } else {
-          atomicExch(err, BT_E_QUEUE_FULL);
-        }
+      for (int j = 0; j < (kLeaves ? leaf_count(v) : 1); j++) {
+        const int slot = (kLeaves ? leaf_slot(v) : v) + j;
+        const TriHit h = test_tri<kP, kCount>(tris, r, rs, dns64, slot, n_tris, hs.limit<kP>(tlim));
+        if (h.ok || h.amb) weigh_hit<kP>(rs, hs.best, slot, h);
       }
-      consider_tri<kP, kCount>(sc, tris, r, rs, dns64, best, kLeaves ? leaf_slot(v) : v, n_tris, tlim);
     }
-    return more;
+  };
+  if (more && (hs.node < 0 || sc.n_tris == 0)) {
+    // nothing to search, or the root of a one-leaf hierarchy
+    if (sc.n_tris > 0 && hs.node != kNoChild) {
+      if (kPairs) expose(hs.node, atomicAdd(wp.n, 1));
+      else test_now(make_int4(hs.node, 0, 0, 0), 1u);
+    }
+    more = false;
   }
-};
-
-// Closest accepted hit of the ray in the BVH under `root`; the leaf slot or -1.
-template <int kP, bool kCount>
-__device__ __forceinline__ int closest_hit(const DevScene &sc, const Ray &r, RaySrc rs, double dns64, Best &best,
-                                           int *err, const WarpCount &n_nodes, const WarpCount &n_tris,
-                                           int root, float tlim = kInf) {
-  // the hot fields in registers: in a batch `sc` lives in device memory and
-  // would otherwise be re-read on every node
-  const int64_t n_tri = sc.n_tris;
-  const Node4 *const nodes = sc.nodes;
-  const Tri *const tris = sc.tris;
-  int stack[kStackDepth];
-  HitSearch hs;
-  hs.start(root);
-  if constexpr (Prec<kP>::defer) rs.pend[0] = 0;
-  while (hs.step<kP, kCount, true>(sc, nodes, tris, n_tri, r, rs, dns64, stack, err, n_nodes, n_tris, tlim)) {
-  }
-  best = hs.best;
-  if constexpr (Prec<kP>::defer) settle_search(sc, r, rs, dns64, best, tlim);
-  return best.slot;
+  unsigned run;
+  do {
+    int4 lc = make_int4(0, 0, 0, 0);
+    unsigned lm = 0;
+    if (more) {
+      if (kCount) n_nodes++;
+      const char *nd = nodes + (size_t)(unsigned)hs.node * sizeof(Node4);
+      // (by address where throughput counts; by value in the split trace, whose
+      // smaller launches wait for the longest chain of fetches, which address
+      // arithmetic lengthens: 81,920 lineages split 4 x 4 1,002 -> 855 us, the
+      // district 38.4 -> 38.0 ms, but the unsplit district 28.9 -> 30.0 ms)
+      const int sx = inv.x < 0.0f ? 16 : 0, sy = inv.y < 0.0f ? 16 : 0, sz = inv.z < 0.0f ? 16 : 0;
+      float4 nx, fx, ny, fy, nz, fz;
+      if (kPairs) {
+        nx = __ldg((const float4 *)(nd + sx)); fx = __ldg((const float4 *)(nd + (sx ^ 16)));
+        ny = __ldg((const float4 *)(nd + 32 + sy)); fy = __ldg((const float4 *)(nd + 32 + (sy ^ 16)));
+        nz = __ldg((const float4 *)(nd + 64 + sz)); fz = __ldg((const float4 *)(nd + 64 + (sz ^ 16)));
+      } else {
+        auto pair = [](const char *p, bool flip, float4 &n, float4 &f) {
+          const float4 lo = __ldg((const float4 *)p), hi = __ldg((const float4 *)(p + 16));
+          n = make_float4(flip ? hi.x : lo.x, flip ? hi.y : lo.y, flip ? hi.z : lo.z, flip ? hi.w : lo.w);
+          f = make_float4(flip ? lo.x : hi.x, flip ? lo.y : hi.y, flip ? lo.z : hi.z, flip ? lo.w : hi.w);
+        };
+        pair(nd, sx != 0, nx, fx);
+        pair(nd + 32, sy != 0, ny, fy);
+        pair(nd + 64, sz != 0, nz, fz);
+      }
+      const int4 ch = __ldg((const int4 *)(nd + 96));
+      const float tmax = hs.limit<kP>(tlim);
+      float k0, k1, k2, k3;
+      const bool h0 = slab_nf(inv, oi, nx.x, fx.x, ny.x, fy.x, nz.x, fz.x, tmax, k0);
+      const bool h1 = slab_nf(inv, oi, nx.y, fx.y, ny.y, fy.y, nz.y, fz.y, tmax, k1);
+      const bool h2 = slab_nf(inv, oi, nx.z, fx.z, ny.z, fy.z, nz.z, fz.z, tmax, k2);
+      const bool h3 = slab_nf(inv, oi, nx.w, fx.w, ny.w, fy.w, nz.w, fz.w, tmax, k3);
+      int c0 = ch.x, c1 = ch.y, c2 = ch.z, c3 = ch.w;
+      const bool l0 = h0 && c0 < 0, l1 = h1 && c1 < 0, l2 = h2 && c2 < 0, l3 = h3 && c3 < 0;
+      if (kPairs) {
+        const int cnt = (int)l0 + (int)l1 + (int)l2 + (int)l3;
+        if (cnt) {
+          int pos = atomicAdd(wp.n, cnt);
+          if (l0) expose(c0, pos++);
+          if (l1) expose(c1, pos++);
+          if (l2) expose(c2, pos++);
+          if (l3) expose(c3, pos);
+        }
+      } else {
+        lc = ch;
+        lm = (unsigned)l0 | (unsigned)l1 << 1 | (unsigned)l2 << 2 | (unsigned)l3 << 3;
+      }
+      // inner children hit, nearest first (a sorting network on the entry
+      // distances; misses sort last)
+      k0 = h0 && !l0 ? k0 : kInf;
+      k1 = h1 && !l1 ? k1 : kInf;
+      k2 = h2 && !l2 ? k2 : kInf;
+      k3 = h3 && !l3 ? k3 : kInf;
+      sort_pair(k0, c0, k1, c1);
+      sort_pair(k2, c2, k3, c3);
+      sort_pair(k0, c0, k2, c2);
+      sort_pair(k1, c1, k3, c3);
+      sort_pair(k1, c1, k2, c2);
+      // a well-formed BVH is visited at most once per node; the bound only
+      // guarantees termination should the structure ever be malformed
+      if (--hs.budget < 0 || hs.sp + 3 > kStackDepth) {
+        atomicExch(err, hs.budget < 0 ? BT_E_TIMEOUT : BT_E_QUEUE_FULL);
+        more = false;
+      } else if (k0 < kInf) {
+        if (k1 < kInf) {
+          if (k2 < kInf) {
+            if (k3 < kInf) stack[hs.sp++] = c3;
+            stack[hs.sp++] = c2;
+          }
+          stack[hs.sp++] = c1;
+        }
+        hs.node = c0;
+      } else if (hs.sp > 0) {
+        hs.node = stack[--hs.sp];
+      } else {
+        more = false;
+      }
+    }
+    if (!kPairs) test_now(lc, lm);
+    run = __ballot_sync(0xffffffffu, more);
+    if (kPairs) {
+      __syncwarp();
+      const int n = *(volatile int *)wp.n;
+      // (the phase's end flushes, so that every lane without nodes is done)
+      if (n >= kPairTest || (n > 0 && __popc(run) <= few))
+        test_pairs<kP, kCount, kLeaves>(wp, n, tris, lane_tris, t_eps, dns, rs, dns64, hs, n_tris, tlim);
+    }
+  } while (__popc(run) > few);
 }
 
-__device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
+// ------------------------------------------------------- groups of lanes
+// Small launches: fewer lineages than the chip has lanes.  Their time is the
+// latency of the longest lineage, one dependent node fetch after the other, so
+// a group of G = 8, 16 or 32 lanes works on one lineage: a step takes the top
+// G / 4 nodes of the group's stack at once, four lanes to a node and one child
+// box to a lane.
+constexpr int kGroupMin = 8;                               // lanes
+constexpr int kGroupCols = kTraceThreads / kGroupMin;      // groups in a block
+// A group takes several nodes a step only while its stack is shallow, so that
+// taking one at a time from there on (at most three more entries per level of
+// the binary hierarchy, kStackDepth in all) still fits.
+constexpr int kGroupShallow = 40;
+constexpr int kGroupDepth = kGroupShallow + 3 * (32 / 4) + kStackDepth;
+constexpr int kGroupPairTest = 8;
+struct GroupStack {
+  int node[kGroupCols][kGroupDepth];
+  unsigned short near[kGroupCols][kGroupDepth];  // upper half of the entry distance's bits (not above it)
+};
+
+// The search phase of a warp whose lanes work in groups of 1 << lg: every
+// group whose leader (lowest lane) has `more` nodes searches to the end.  rs
+// points at the group's column and r holds its ray in all of its lanes (r.dns,
+// dns64, hs, more and tlim count in the leader).  Warp-collective.
+template <int kP>
+__device__ __forceinline__ void search_groups(const DevScene &sc, bool lane_tris, const Ray &r, const RaySrc &rs,
+                                              double dns64, int *near_node, unsigned short *near_dist, int *err,
+                                              HitSearch &hs, bool &more, const WarpPairs &wp, const WarpCount &n_tris,
+                                              float tlim, int lg) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = (int)lane_id(), G = 1 << lg;
+  const int leader = lane & ~(G - 1), sub = lane & 3, q = (lane & (G - 1)) >> 2;
+  const unsigned group = G == 32 ? kAll : (1u << G) - 1u;
+  const Tri *const tris = sc.tris;
+  const float3 inv = r.inv, oi = origin_scaled(r);
+  const char *const nodes = (const char *)sc.nodes + 4 * sub;
+  int root = hs.node, n = 0;
+  if (!more || sc.n_tris == 0) root = kNoChild;
+  {
+    // the root of a one-leaf hierarchy
+    const bool leaf = root < 0 && root != kNoChild;
+    const unsigned lb = __ballot_sync(kAll, leaf);
+    if (leaf) {
+      const int pos = __popc(lb & ((1u << lane) - 1u));
+      wp.code[pos] = ~root;
+      wp.lane[pos] = (unsigned char)lane;
+    }
+    n = __popc(lb);
+  }
+  root = __shfl_sync(kAll, root, leader);
+  int sp = root >= 0 ? 1 : 0;  // (the same in all lanes of the group)
+  if (sp && lane == leader) {
+    near_node[0] = root;
+    near_dist[0] = 0;
+  }
+  unsigned run = __ballot_sync(kAll, sp > 0);
+  __syncwarp();
+  while (run != 0u || n > 0) {
+    if (run != 0u) {
+      const float tmax = __shfl_sync(kAll, hs.limit<kP>(tlim), leader);
+      // this step's nodes: the top `take` of the stack, the nearest first
+      const int take = min(sp, sp <= kGroupShallow ? G >> 2 : 1);
+      const int at = sp - 1 - q;
+      bool hit = false;
+      int code = kNoChild;
+      float tn = kInf;
+      if (q < take && __uint_as_float((unsigned)near_dist[at] << 16) <= tmax) {
+        const char *nd = nodes + (size_t)(unsigned)near_node[at] * sizeof(Node4);
+        const float lx = __ldg((const float *)nd), hx = __ldg((const float *)(nd + 16));
+        const float ly = __ldg((const float *)(nd + 32)), hy = __ldg((const float *)(nd + 48));
+        const float lz = __ldg((const float *)(nd + 64)), hz = __ldg((const float *)(nd + 80));
+        code = __ldg((const int *)(nd + 96));
+        const bool sx = inv.x < 0.0f, sy = inv.y < 0.0f, sz = inv.z < 0.0f;
+        hit = slab_nf(inv, oi, sx ? hx : lx, sx ? lx : hx, sy ? hy : ly, sy ? ly : hy, sz ? hz : lz, sz ? lz : hz,
+                      tmax, tn);
+      }
+      const bool leaf = hit && code < 0, inner = hit && code >= 0;
+      const unsigned lb = __ballot_sync(kAll, leaf), ib = (__ballot_sync(kAll, inner) >> leader) & group;
+      if (leaf) {
+        const int pos = n + __popc(lb & ((1u << lane) - 1u));
+        wp.code[pos] = ~code;
+        wp.lane[pos] = (unsigned char)leader;
+      }
+      n += __popc(lb);
+      // the inner children hit: the nearest node's on top, nearest first
+      const unsigned key = inner ? (__float_as_uint(tn) & ~3u) | (unsigned)sub : ~0u;
+      const int rank = (int)(__shfl_xor_sync(kAll, key, 1) < key) + (int)(__shfl_xor_sync(kAll, key, 2) < key) +
+                       (int)(__shfl_xor_sync(kAll, key, 3) < key);
+      const int total = __popc(ib);
+      sp += total - take;
+      // a well-formed BVH is visited at most once per node; the bound only
+      // guarantees termination should the structure ever be malformed
+      if (sp > kGroupDepth || __shfl_sync(kAll, hs.budget -= take, leader) < 0) {
+        if (lane == leader) atomicExch(err, sp > kGroupDepth ? BT_E_QUEUE_FULL : BT_E_TIMEOUT);
+        sp = 0;
+      } else if (inner) {
+        const int to = sp - 1 - (__popc(ib & ((1u << (4 * q)) - 1u)) + rank);
+        near_node[to] = code;
+        near_dist[to] = (unsigned short)(__float_as_uint(tn) >> 16);
+      }
+      run = __ballot_sync(kAll, sp > 0);
+      __syncwarp();
+    }
+    if (n >= kGroupPairTest || (run == 0u && n > 0)) {
+      test_pairs<kP, false, false>(wp, n, tris, lane_tris, r.t_eps, r.dns, rs, dns64, hs, n_tris, tlim, lg);
+      n = 0;
+    }
+  }
+  more = false;
+}
 
 // Cheap rejection of a segment that cannot reach the microphones' height
 // slab: the cone lies on one side of its apex height when all three edge
@@ -547,25 +806,25 @@ __device__ __forceinline__ void emit_segment(const TraceArgs &a, const Seg &s, b
 // that it holds no registers across the traversal.  Rows: apex 0..2, cone
 // normals 3..11, ray origin 12..14, ray direction 15..17; `lo` holds the low
 // parts of the float pairs (MIXED only).
-constexpr int kTraceThreads = 128;
 
 constexpr int kRowA = 0, kRowN = 3, kRowO = 12, kRowD = 15, kRows = 18;
 // a sub-domain accepts hits up to this far (m along the ray) past its exit
 constexpr float kTileEps = 1e-2f;
 // per-lane event counters (rows of LineageSmem::cnt)
 enum { kCSeg, kCHit, kCEsc, kCEmit, kCHand, kCSteal, kCNodes, kCTris, kNumCounts };
-template <int kP>
+// kC columns, one per lineage a block holds.
+template <int kP, int kC>
 struct LineageSmem {
-  double dv[Prec<kP>::chain64 ? kRows : 1][kTraceThreads];  // float64 chain; `hi` holds its float32 rounding
-  float hi[kRows][kTraceThreads];
-  float lo[Prec<kP>::pairs ? kRows : 1][kTraceThreads];
-  float p[kMaxBands][kTraceThreads];  // band power W_b prod(r_b)
-  float st[4][kTraceThreads];         // start plane (relative to the apex)
-  int pend[Prec<kP>::defer ? kPend + 1 : 1][kTraceThreads];  // candidates left to float64
+  double dv[Prec<kP>::chain64 ? kRows : 1][Prec<kP>::chain64 ? kC : 1];  // float64 chain; `hi` holds its float32 rounding
+  float hi[kRows][kC];
+  float lo[Prec<kP>::pairs ? kRows : 1][Prec<kP>::pairs ? kC : 1];
+  float p[kMaxBands][kC];  // band power W_b prod(r_b)
+  float st[4][kC];         // start plane (relative to the apex)
+  int pend[Prec<kP>::defer ? kPend + 1 : 1][Prec<kP>::defer ? kC : 1];  // candidates left to float64
 };
 
-template <int kP>
-__device__ __forceinline__ df3 ld_df3(const LineageSmem<kP> &sm, int row, int t) {
+template <int kP, int kC>
+__device__ __forceinline__ df3 ld_df3(const LineageSmem<kP, kC> &sm, int row, int t) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   df3 v;
   v.x = df{sm.hi[row][t], kPairs ? sm.lo[row][t] : 0.0f};
@@ -573,8 +832,8 @@ __device__ __forceinline__ df3 ld_df3(const LineageSmem<kP> &sm, int row, int t)
   v.z = df{sm.hi[row + 2][t], kPairs ? sm.lo[row + 2][t] : 0.0f};
   return v;
 }
-template <int kP>
-__device__ __forceinline__ void st_df3(LineageSmem<kP> &sm, int row, int t, df3 v) {
+template <int kP, int kC>
+__device__ __forceinline__ void st_df3(LineageSmem<kP, kC> &sm, int row, int t, df3 v) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   sm.hi[row][t] = v.x.hi;
   sm.hi[row + 1][t] = v.y.hi;
@@ -585,13 +844,13 @@ __device__ __forceinline__ void st_df3(LineageSmem<kP> &sm, int row, int t, df3 
     sm.lo[row + 2][t] = v.z.lo;
   }
 }
-template <int kP>
-__device__ __forceinline__ float3 ld_hi3(const LineageSmem<kP> &sm, int row, int t) {
+template <int kP, int kC>
+__device__ __forceinline__ float3 ld_hi3(const LineageSmem<kP, kC> &sm, int row, int t) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   return make_float3(sm.hi[row][t], sm.hi[row + 1][t], sm.hi[row + 2][t]);
 }
-template <int kP>
-__device__ __forceinline__ void st_f3(LineageSmem<kP> &sm, int row, int t, float3 v) {
+template <int kP, int kC>
+__device__ __forceinline__ void st_f3(LineageSmem<kP, kC> &sm, int row, int t, float3 v) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   sm.hi[row][t] = v.x;
   sm.hi[row + 1][t] = v.y;
@@ -600,12 +859,12 @@ __device__ __forceinline__ void st_f3(LineageSmem<kP> &sm, int row, int t, float
 
 // FP64 rows: the float64 value and its float32 rounding in `hi` (read by the
 // float32 traversal and the segment records).
-template <int kP>
-__device__ __forceinline__ double3 ld_d3(const LineageSmem<kP> &sm, int row, int t) {
+template <int kP, int kC>
+__device__ __forceinline__ double3 ld_d3(const LineageSmem<kP, kC> &sm, int row, int t) {
   return make_double3(sm.dv[row][t], sm.dv[row + 1][t], sm.dv[row + 2][t]);
 }
-template <int kP>
-__device__ __forceinline__ void st_d3(LineageSmem<kP> &sm, int row, int t, double3 v) {
+template <int kP, int kC>
+__device__ __forceinline__ void st_d3(LineageSmem<kP, kC> &sm, int row, int t, double3 v) {
   sm.dv[row][t] = v.x;
   sm.dv[row + 1][t] = v.y;
   sm.dv[row + 2][t] = v.z;
@@ -615,8 +874,8 @@ __device__ __forceinline__ void st_d3(LineageSmem<kP> &sm, int row, int t, doubl
 }
 
 // Start lineage `lin` (source si, beam bi) in this thread's column.
-template <int kP>
-__device__ __forceinline__ void init_lineage(const SceneView &a, LineageSmem<kP> &sm, int t, int64_t lin) {
+template <int kP, int kC>
+__device__ __forceinline__ void init_lineage(const SceneView &a, LineageSmem<kP, kC> &sm, int t, int64_t lin) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   const int nb = a.sc.n_bands;
   int64_t si = lin / a.n_beams, bi = lin - si * a.n_beams;
@@ -697,8 +956,8 @@ __device__ __forceinline__ TraceCounts init_counts(unsigned (*wc)[kNumCounts], i
 // < 0).  Write the segment record and, if the beam goes on, reflect it: the
 // image source (Section 2), mirrored cone and axis, energy lost at the
 // reflection.  Returns true if the lineage continues.
-template <int kP>
-__device__ __forceinline__ bool finish_segment(const TraceArgs &a, const SceneView &v, int vi, LineageSmem<kP> &sm,
+template <int kP, int kC>
+__device__ __forceinline__ bool finish_segment(const TraceArgs &a, const SceneView &v, int vi, LineageSmem<kP, kC> &sm,
                                                int t, const Ray &r, const Best &best, int slot, LaneState &ls,
                                                const TraceCounts &cn) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
@@ -977,36 +1236,47 @@ constexpr int kRefillLanes = 28;
 // scenes (views) in one launch, each lane on its own lineage's scene.
 //
 // Each warp alternates two phases.  In the search phase every lane with a ray
-// steps through the BVH one node at a time; the phase ends once kRefillLanes
-// lanes have nothing to search (their search finished, or they need a new
-// lineage) or no lane is searching.  In the service phase, reconverged, the
+// steps through the BVH one node at a time and the warp tests the triangles
+// they expose (by pairs: district unsplit 32.8 -> 29.0 ms together with the
+// near/far slab test and the wider-first nodes, FP64 on 24 of its sources
+// 8.4 -> 4.8 ms a call); the phase ends once kRefillLanes lanes have nothing to
+// search (their search finished, or they need a new lineage) or no lane is
+// searching.  In the service phase, reconverged, the
 // lanes whose search finished write their segment and reflect (or end their
 // lineage), lanes without a lineage take new ones, and new searches start --
 // while the lanes still searching keep their state, so a long search no longer
 // holds the whole warp (dynamic ray fetch, after Aila & Laine 2009).
-template <int kP, bool kCount, bool kBatch, bool kLeaves>
+template <int kP, bool kCount, bool kBatch, bool kLeaves, bool kGroup>
 __global__ void __launch_bounds__(kTraceThreads, kP == kPMixed && !kBatch ? 7 : 6) k_trace(TraceArgs a) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
-  __shared__ LineageSmem<kP> sm;
+  __shared__ LineageSmem<kP, kGroup ? kGroupCols : kTraceThreads> sm;
+  __shared__ typename std::conditional<kGroup, GroupStack, char>::type gstack;
   __shared__ int64_t view_base[kBatch ? BT_MAX_SCENES : 1];
   __shared__ WarpLineages wlin[kTraceThreads / 32];
-  const int t = threadIdx.x;
-  if ((t & 31) == 0) wlin[t >> 5] = WarpLineages{0ull, 0ull, 0};
+  // kGroup: lanes work in groups of 1 << lg, each on one lineage (column t)
+  const int lg = kGroup ? a.group_log2 : 0;
+  const int t = (int)threadIdx.x >> lg;
+  const int warp = (int)threadIdx.x >> 5;
+  if (lane_id() == 0) wlin[warp] = WarpLineages{0ull, 0ull, 0};
   __syncwarp();
   if (kBatch) {
-    for (int i = t; i < a.n_views; i += kTraceThreads) view_base[i] = a.views[i].lineage_base;
+    for (int i = threadIdx.x; i < a.n_views; i += kTraceThreads) view_base[i] = a.views[i].lineage_base;
     __syncthreads();
   }
   __shared__ unsigned wcount[kTraceThreads / 32][kNumCounts];
-  const TraceCounts cn = init_counts(wcount, t);
+  const TraceCounts cn = init_counts(wcount, threadIdx.x);
   LaneState ls = {-1, 0, -1, 0.0f, 0.0};
   int vi = 0;  // this lane's scene view
-  bool done = false, searching = false, pending = false;
+  __shared__ PairQueue<kTraceThreads / 32> pairs;
+  const WarpPairs wp = warp_pairs(pairs);
+  bool done = (lane_id() & ((1u << lg) - 1u)) != 0;  // (only a group's leader takes lineages)
+  bool more = false;        // its search has nodes left to visit
+  bool pending = false;     // its search is over and awaits service
   HitSearch hs;
-  hs.start(-1);
-  int stack[kStackDepth];
-  const RaySrc rs{&sm.hi[kRowO][t], kPairs ? &sm.lo[kRowO][t] : &sm.hi[kRowO][t], kTraceThreads,
-                  kChain64 ? &sm.dv[kRowO][t] : nullptr, &sm.pend[0][t]};
+  hs.start(-1, 0);
+  int stack[kGroup ? 1 : kStackDepth];
+  const RaySrc rs{&sm.hi[kRowO][t], kPairs ? &sm.lo[kRowO][t] : &sm.hi[kRowO][t], kGroup ? kGroupCols : kTraceThreads,
+                  kChain64 ? &sm.dv[kRowO][t] : nullptr, kDefer ? &sm.pend[0][t] : nullptr};
   while (true) {
     // ---- service: finished searches write their segment and reflect
     bool fresh = false;
@@ -1020,7 +1290,7 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPMixed && !kBatch ? 7 : 
     }
     // ---- service: lanes without a lineage take the next ones
     bool need = !done && ls.lin < 0;
-    int64_t mine = take_lineage(a, need, wlin[t >> 5]);
+    int64_t mine = take_lineage(a, need, wlin[warp]);
     if (need) {
       if (mine >= 0) {
         if (kBatch) {
@@ -1035,29 +1305,32 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPMixed && !kBatch ? 7 : 
       }
     }
     if (fresh) {
-      hs.start((kBatch ? a.views[vi] : a.v).sc.root);
+      const DevScene &fs = (kBatch ? a.views[vi] : a.v).sc;
+      hs.start(fs.root, fs.n_tris);
       if constexpr (kDefer) rs.pend[0] = 0;
-      searching = true;
+      more = true;
     }
     if (__all_sync(0xffffffffu, done)) break;
     // ---- search
     {
+      if constexpr (kGroup) {
+        // (the group's other lanes read the ray its leader has just written)
+        vi = __shfl_sync(0xffffffffu, vi, (int)lane_id() & ~((1 << lg) - 1));
+        __syncwarp();
+      }
       const SceneView &v = kBatch ? a.views[vi] : a.v;
       const Ray r = make_ray(ld_hi3(sm, kRowO, t), ld_hi3(sm, kRowD, t), v.t_eps, ls.dns);
-      const int64_t n_tri = v.sc.n_tris;
-      const Node4 *const nodes = v.sc.nodes;
-      const Tri *const tris = v.sc.tris;
-      while (true) {
-        if (searching &&
-            !hs.step<kP, kCount, kLeaves>(v.sc, nodes, tris, n_tri, r, rs, ls.dns64, stack, &a.ctr->error,
-                                          cn[kCNodes], cn[kCTris], kInf)) {
-          searching = false;
-          pending = true;
-        }
-        const unsigned srch = __ballot_sync(0xffffffffu, searching);
-        const unsigned idle = __ballot_sync(0xffffffffu, !searching && !done);
-        if (!srch || __popc(idle) >= kRefillLanes) break;
+      const bool searching = more;
+      const int few = max(0, 32 - kRefillLanes - __popc(__ballot_sync(0xffffffffu, done)));
+      if constexpr (kGroup) {
+        search_groups<kP>(v.sc, kBatch, r, rs, ls.dns64, gstack.node[t], gstack.near[t], &a.ctr->error, hs, more, wp,
+                          cn[kCTris], kInf, lg);
+        pending = searching;
+        continue;
       }
+      search_phase<kP, kCount, kLeaves, true>(v.sc, kBatch, r, rs, ls.dns64, stack, &a.ctr->error, hs, more, wp, cn[kCNodes],
+                                        cn[kCTris], kInf, few);
+      pending = searching && !more;
     }
   }
   flush_counts(a, cn, kCount);
@@ -1100,8 +1373,8 @@ __device__ __forceinline__ bool wait_slot(const TraceArgs &a, const TiledArgs &t
 // A lineage's state in a queue slot: S points at row 0, rows c words apart.
 // Queue slots are written once and read once by another SM, so both sides
 // go through L2 only.
-template <int kP>
-__device__ __forceinline__ void save_state(uint32_t *S, size_t c, const LineageSmem<kP> &sm, int t,
+template <int kP, int kC>
+__device__ __forceinline__ void save_state(uint32_t *S, size_t c, const LineageSmem<kP, kC> &sm, int t,
                                            const LaneState &ls) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   if (kChain64) {
@@ -1128,8 +1401,8 @@ __device__ __forceinline__ void save_state(uint32_t *S, size_t c, const LineageS
   __stcg(S + 54 * c, (uint32_t)(d >> 32));
 }
 
-template <int kP>
-__device__ __forceinline__ void load_state(const uint32_t *S, size_t c, LineageSmem<kP> &sm, int t,
+template <int kP, int kC>
+__device__ __forceinline__ void load_state(const uint32_t *S, size_t c, LineageSmem<kP, kC> &sm, int t,
                                            LaneState &ls) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
   if (kChain64) {
@@ -1277,6 +1550,14 @@ __device__ __forceinline__ int take_fresh(const TraceArgs &a, const TiledArgs &t
 // 65.0 ms at 28 on the district with 4x4 sub-domains).
 constexpr int kRefillTiled = 32;
 
+// Whether the split trace tests triangles by pairs: in FP64, whose triangle
+// test is long (a whole-warp float64 instruction costs the same for 4 lanes as
+// for 32).  In the other variants the pairs' code, added to the queue code, no
+// longer fits the instruction cache beside it (no-instruction stalls 0.9 -> 2.8
+// cycles per issue): 44.1 ms against 37.4 ms on the district split 4x4.
+template <int kP>
+constexpr bool kTilePairs = kP == kPF64;
+
 // Distance along r to its exit from tile (ix, iy) of the grid, in the xy plane.
 __device__ __forceinline__ float tile_exit(const TileGrid &tg, int ix, int iy, const Ray &r) {
   float tex = kInf, tey = kInf;
@@ -1310,17 +1591,21 @@ __device__ __forceinline__ float tile_exit(const TileGrid &tg, int ix, int iy, c
 // whose smaller state fits them (40.7 -> 38.3 ms on the district split 4x4),
 // and for MIXED (39.8 against 40.7 ms at six); six for the float64-chain
 // variants.
-template <int kP, bool kCount, bool kLeaves>
+template <int kP, bool kCount, bool kLeaves, bool kGroup>
 __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 7 : 6) k_trace_tiled(TraceArgs a, const __grid_constant__ TiledArgs ta) {
   [[maybe_unused]] constexpr bool kPairs = Prec<kP>::pairs, kChain64 = Prec<kP>::chain64, kDefer = Prec<kP>::defer;
-  __shared__ LineageSmem<kP> sm;
-  const int t = threadIdx.x;
+  __shared__ LineageSmem<kP, kGroup ? kGroupCols : kTraceThreads> sm;
+  __shared__ typename std::conditional<kGroup, GroupStack, char>::type gstack;
+  // kGroup: lanes work in groups of 1 << lg, each on one lineage (column t)
+  const int lg = kGroup ? a.group_log2 : 0;
+  const int t = (int)threadIdx.x >> lg;
   const unsigned lane = lane_id();
+  const bool lead = (lane & ((1u << lg) - 1u)) == 0u;  // (only a group's leader takes lineages)
   const unsigned below = (1u << lane) - 1u;
   const SceneView &v = a.v;
   const TileGrid &tg = ta.tg;  // read from parameter space, not held in registers
   __shared__ unsigned wcount[kTraceThreads / 32][kNumCounts];
-  const TraceCounts cn = init_counts(wcount, t);
+  const TraceCounts cn = init_counts(wcount, threadIdx.x);
   const size_t qc = ta.qcap;
   const unsigned qmask = ta.qcap - 1u;
   int *const used = ta.ctl + 3 * ta.n_tiles;
@@ -1332,7 +1617,9 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
   __syncwarp();
   LaneState ls = {-1, 0, -1, 0.0f, 0.0};
   bool active = false;      // the lane holds a lineage
-  bool searching = false;   // its search in the current tile is under way
+  __shared__ PairQueue<kTraceThreads / 32> pairs;
+  const WarpPairs wp = warp_pairs(pairs);
+  bool more = false;        // its search has nodes left to visit
   bool pending = false;     // its search is over and awaits service
   int tile = -1;
   float tlim = kInf;        // hits are accepted up to this distance
@@ -1340,10 +1627,10 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
   const int home = (int)((blockIdx.x * (kTraceThreads / 32) + (threadIdx.x >> 5)) % (unsigned)ta.n_tiles);
   unsigned long long idle_since = 0, last_prog = 0;
   HitSearch hs;
-  hs.start(-1);
-  int stack[kStackDepth];
-  const RaySrc rs{&sm.hi[kRowO][t], kPairs ? &sm.lo[kRowO][t] : &sm.hi[kRowO][t], kTraceThreads,
-                  kChain64 ? &sm.dv[kRowO][t] : nullptr, &sm.pend[0][t]};
+  hs.start(-1, 0);
+  int stack[kGroup ? 1 : kStackDepth];
+  const RaySrc rs{&sm.hi[kRowO][t], kPairs ? &sm.lo[kRowO][t] : &sm.hi[kRowO][t], kGroup ? kGroupCols : kTraceThreads,
+                  kChain64 ? &sm.dv[kRowO][t] : nullptr, kDefer ? &sm.pend[0][t] : nullptr};
   while (true) {
     // ---- service: finished searches write their segment and reflect, end,
     // or go on to the next tile
@@ -1428,12 +1715,12 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
       active = false;
     }
     // ---- refill: hand-offs first (home tile, then steals), then fresh lineages
-    unsigned nm = __ballot_sync(0xffffffffu, !active);
+    unsigned nm = __ballot_sync(0xffffffffu, lead && !active);
     if (nm) {
       unsigned base;
       int got;
       int qt = take_handoffs(ta, home, __popc(nm), base, got);
-      if (qt >= 0 && !active) {
+      if (qt >= 0 && lead && !active) {
         int rank = __popc(nm & below);
         if (rank < got) {
           unsigned pos = base + (unsigned)rank, gen = pos & ~qmask, slot = pos & qmask;
@@ -1450,12 +1737,12 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
           }
         }
       }
-      nm = __ballot_sync(0xffffffffu, !active);
+      nm = __ballot_sync(0xffffffffu, lead && !active);
       if (nm && !exhausted) {
         int64_t fb;
         int got_f = take_fresh(a, ta, __popc(nm), credits, fb, exhausted, wlin[threadIdx.x >> 5]);
         int rank = __popc(nm & below);
-        if (!active && rank < got_f) {
+        if (lead && !active && rank < got_f) {
           int64_t mine = a.lineage_begin + fb + rank;
           ls = LaneState{mine, 0, -1, 0.0f, 0.0};
           init_lineage(v, sm, t, mine);
@@ -1473,9 +1760,9 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
       // is the ray's first, and a ray with none goes on to the next tile.
       const Ray r = make_ray(ld_hi3(sm, kRowO, t), ld_hi3(sm, kRowD, t), v.t_eps, ls.dns);
       tlim = tile_exit(tg, tile % tg.tx, tile / tg.tx, r) + kTileEps;
-      hs.start(__ldg(&ta.roots[tile]));
+      hs.start(__ldg(&ta.roots[tile]), v.sc.n_tris);
       if constexpr (kDefer) rs.pend[0] = 0;
-      searching = true;
+      more = true;
     }
     if (!__any_sync(0xffffffffu, active)) {
       // nothing to trace: done once every lineage of the batch has finished
@@ -1501,42 +1788,76 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
     // or no lineage while fresh ones remain) or no lane is searching
     {
       const Ray r = make_ray(ld_hi3(sm, kRowO, t), ld_hi3(sm, kRowD, t), v.t_eps, ls.dns);
-      const int64_t n_tri = v.sc.n_tris;
-      const Node4 *const nodes = v.sc.nodes;
-      const Tri *const tris = v.sc.tris;
-      while (true) {
-        if (searching && !hs.step<kP, kCount, kLeaves>(v.sc, nodes, tris, n_tri, r, rs, ls.dns64, stack,
-                                                       &a.ctr->error, cn[kCNodes], cn[kCTris], tlim)) {
-          searching = false;
-          pending = true;
-        }
-        const unsigned srch = __ballot_sync(0xffffffffu, searching);
-        const unsigned idle = __ballot_sync(0xffffffffu, pending || (!active && !exhausted));
-        if (!srch || __popc(idle) >= kRefillTiled) break;
+      const bool searching = more;
+      if constexpr (kGroup) {
+        __syncwarp();
+        const Ray r = make_ray(ld_hi3(sm, kRowO, t), ld_hi3(sm, kRowD, t), v.t_eps, ls.dns);
+        search_groups<kP>(v.sc, false, r, rs, ls.dns64, gstack.node[t], gstack.near[t], &a.ctr->error, hs, more, wp,
+                          cn[kCTris], tlim, lg);
+        pending = searching;
+        continue;
       }
+      const int few = max(0, 32 - kRefillTiled - __popc(__ballot_sync(0xffffffffu, !active && exhausted)));
+      search_phase<kP, kCount, kLeaves, kTilePairs<kP>>(v.sc, false, r, rs, ls.dns64, stack, &a.ctr->error, hs, more, wp, cn[kCNodes],
+                                        cn[kCTris], tlim, few);
+      pending = searching && !more;
     }
   }
   flush_counts(a, cn, kCount);
 }
 
-template <int kP, bool kCount, bool kLeaves>
+// Lanes that work on one lineage, as a power of two, for a launch of n
+// lineages: 16 or 8 while the chip's lanes (seven blocks per SM) are enough to
+// give every lineage some, which its chain of dependent fetches needs more than
+// the launch needs throughput.  Measured (trace kernel, us, 1 / 8 / 16 / 32
+// lanes per lineage; district and an 8 x 8-block city, order 4, MIXED):
+//   lineages   5,120  159/83/73/77 and 139/74/66/79
+//             10,240  245/123/107/132 and 146/79/86/131
+//             40,960  317/214/277/445 and 166/159/225/368
+//             61,440  328/299/406/674 and 202/212/309/511
+// split 4 x 4: 5,120 385/333/336/352, 40,960 968/634/767/966.  Not for the
+// float64 chain, which leaves too much to one lane of a group (FP64 at 10,240
+// lineages 344/245/332/541 and 225/249/374/623).
+template <int kP>
+static int group_log2(int64_t n, int n_sm) {
+  const int64_t lanes = (int64_t)n_sm * 7 * kTraceThreads;
+  if (Prec<kP>::chain64) return 0;
+  return n <= lanes / 16 ? 4 : (n <= lanes * 3 / 8 ? 3 : 0);
+}
+
+template <int kP, bool kCount, bool kLeaves, bool kGroup>
 static cudaError_t launch_tiled_t(cudaStream_t st, const TraceArgs &a, const TiledArgs &ta, int n_sm) {
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_tiled<kP, kCount, kLeaves>,
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_tiled<kP, kCount, kLeaves, kGroup>,
                                                                 kTraceThreads, 0);
   if (e != cudaSuccess) return e;
   if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
   if (per_sm < 1) per_sm = 1;
   int64_t blocks = (int64_t)n_sm * per_sm;
-  k_trace_tiled<kP, kCount, kLeaves><<<(int)blocks, kTraceThreads, 0, st>>>(a, ta);
+  if (kGroup) {
+    // no more blocks than lineages need: warps without work poll the queues,
+    // which slows a small launch down (5,120 lineages split 4 x 4: 262 -> 190 us)
+    const int cols = kTraceThreads >> a.group_log2;
+    const int64_t need = (a.lineage_end - a.lineage_begin + cols - 1) / cols;
+    if (blocks > need) blocks = need;
+  }
+  k_trace_tiled<kP, kCount, kLeaves, kGroup><<<(int)blocks, kTraceThreads, 0, st>>>(a, ta);
   return cudaGetLastError();
 }
 
 template <int kP>
-static cudaError_t launch_tiled_p(cudaStream_t st, const TraceArgs &a, const TiledArgs &ta, int n_sm) {
+static cudaError_t launch_tiled_p(cudaStream_t st, const TraceArgs &a0, const TiledArgs &ta, int n_sm) {
+  TraceArgs a = a0;
+  a.group_log2 = group_log2<kP>(a.lineage_end - a.lineage_begin, n_sm);
   if (a.leaf_size > 1)
-    return a.count_work ? launch_tiled_t<kP, true, true>(st, a, ta, n_sm) : launch_tiled_t<kP, false, true>(st, a, ta, n_sm);
-  return a.count_work ? launch_tiled_t<kP, true, false>(st, a, ta, n_sm) : launch_tiled_t<kP, false, false>(st, a, ta, n_sm);
+    return a.count_work ? launch_tiled_t<kP, true, true, false>(st, a, ta, n_sm)
+                        : launch_tiled_t<kP, false, true, false>(st, a, ta, n_sm);
+  if (a.count_work) return launch_tiled_t<kP, true, false, false>(st, a, ta, n_sm);
+  // (FP32's chain rounds by each kernel's own contractions, so it keeps to the
+  // kernel that larger launches run)
+  if constexpr (kP == kPMixed)
+    if (a.group_log2 > 0) return launch_tiled_t<kP, false, false, true>(st, a, ta, n_sm);
+  return launch_tiled_t<kP, false, false, false>(st, a, ta, n_sm);
 }
 
 cudaError_t launch_trace_tiled(cudaStream_t st, const TraceArgs &a, const TiledArgs &ta, int n_sm) {
@@ -1551,7 +1872,7 @@ cudaError_t launch_trace_tiled(cudaStream_t st, const TraceArgs &a, const TiledA
 
 int tiled_resident_lanes(int n_sm) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_tiled<kPMixed, false, false>, kTraceThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_tiled<kPMixed, false, false, false>, kTraceThreads, 0) !=
       cudaSuccess)
     per_sm = 8;
   if (per_sm < 1) per_sm = 1;
@@ -1566,23 +1887,37 @@ __global__ void __launch_bounds__(128) k_cast(DevScene sc, const float *o, const
                                               int64_t n, float t_eps, float *t_out, int *tri_out, int *err) {
   __shared__ float rh[6][128], rl[6][128];
   __shared__ int pend[kPend + 1][128];
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  __shared__ PairQueue<4> pairs;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool mine = i < n;  // (a warp's lanes search together, so none returns early)
   const int t = threadIdx.x;
-  float3 O = make_float3(o[3 * i], o[3 * i + 1], o[3 * i + 2]);
-  double3 Dd = normalize3(make_double3(d[3 * i], d[3 * i + 1], d[3 * i + 2]));
-  df3 D = df3{d_to_df(Dd.x), d_to_df(Dd.y), d_to_df(Dd.z)};
+  float3 O = make_float3(0.0f, 0.0f, 0.0f);
+  double3 Dd = make_double3(0.0, 0.0, 1.0);
   double dns = 0.0;
-  if (ns) dns = fabs(dot3(Dd, make_double3(ns[3 * i], ns[3 * i + 1], ns[3 * i + 2])));
+  if (mine) {
+    O = make_float3(o[3 * i], o[3 * i + 1], o[3 * i + 2]);
+    Dd = normalize3(make_double3(d[3 * i], d[3 * i + 1], d[3 * i + 2]));
+    if (ns) dns = fabs(dot3(Dd, make_double3(ns[3 * i], ns[3 * i + 1], ns[3 * i + 2])));
+  }
+  df3 D = df3{d_to_df(Dd.x), d_to_df(Dd.y), d_to_df(Dd.z)};
   rh[0][t] = O.x; rh[1][t] = O.y; rh[2][t] = O.z;
   rl[0][t] = 0.0f; rl[1][t] = 0.0f; rl[2][t] = 0.0f;
   rh[3][t] = D.x.hi; rh[4][t] = D.y.hi; rh[5][t] = D.z.hi;
   rl[3][t] = D.x.lo; rl[4][t] = D.y.lo; rl[5][t] = D.z.lo;
+  pend[0][t] = 0;
   Ray r = make_ray(O, df3_hi(D), t_eps, (float)dns);
-  Best best;
-  const WarpCount a{nullptr}, b{nullptr};
+  const WarpCount none{nullptr};
   const RaySrc rs{&rh[0][t], &rl[0][t], 128, nullptr, &pend[0][t]};
-  int slot = closest_hit<kPMixed, false>(sc, r, rs, dns, best, err, a, b, sc.root);
+  const WarpPairs wp = warp_pairs(pairs);
+  int stack[kStackDepth];
+  HitSearch hs;
+  hs.start(sc.root, sc.n_tris);
+  bool more = mine;
+  search_phase<kPMixed, false, true, true>(sc, false, r, rs, dns, stack, err, hs, more, wp, none, none, kInf, 0);
+  if (!mine) return;
+  Best &best = hs.best;
+  settle_search(sc, r, rs, dns, best, kInf);
+  const int slot = best.slot;
   // the reported distance is the float64 one to the hit triangle's plane
   // along the float-pair ray (the search itself decides in float32)
   double t64 = best.t64;
@@ -1605,29 +1940,34 @@ cudaError_t launch_cast(cudaStream_t st, const DevScene &sc, const float *o, con
 
 // One persistent grid: enough blocks to fill every SM at the kernel's
 // occupancy, each block looping until the batch's lineages are taken.
-template <int kP, bool kCount, bool kBatch, bool kLeaves>
+template <int kP, bool kCount, bool kBatch, bool kLeaves, bool kGroup>
 static cudaError_t launch_trace_t(cudaStream_t st, const TraceArgs &a, int n_sm) {
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace<kP, kCount, kBatch, kLeaves>,
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace<kP, kCount, kBatch, kLeaves, kGroup>,
                                                                 kTraceThreads, 0);
   if (e != cudaSuccess) return e;
   if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
   if (per_sm < 1) per_sm = 1;
   int64_t n = a.lineage_end - a.lineage_begin;
   int64_t blocks = (int64_t)n_sm * per_sm;
-  int64_t need = (n + kTraceThreads - 1) / kTraceThreads;
+  const int cols = kTraceThreads >> (kGroup ? a.group_log2 : 0);
+  int64_t need = (n + cols - 1) / cols;
   if (blocks > need) blocks = need;
-  k_trace<kP, kCount, kBatch, kLeaves><<<(int)blocks, kTraceThreads, 0, st>>>(a);
+  k_trace<kP, kCount, kBatch, kLeaves, kGroup><<<(int)blocks, kTraceThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 template <int kP, bool kBatch>
-static cudaError_t launch_trace_p(cudaStream_t st, const TraceArgs &a, int n_sm) {
+static cudaError_t launch_trace_p(cudaStream_t st, const TraceArgs &a0, int n_sm) {
+  TraceArgs a = a0;
+  a.group_log2 = group_log2<kP>(a.lineage_end - a.lineage_begin, n_sm);
   if (a.leaf_size > 1)
-    return a.count_work ? launch_trace_t<kP, true, kBatch, true>(st, a, n_sm)
-                        : launch_trace_t<kP, false, kBatch, true>(st, a, n_sm);
-  return a.count_work ? launch_trace_t<kP, true, kBatch, false>(st, a, n_sm)
-                      : launch_trace_t<kP, false, kBatch, false>(st, a, n_sm);
+    return a.count_work ? launch_trace_t<kP, true, kBatch, true, false>(st, a, n_sm)
+                        : launch_trace_t<kP, false, kBatch, true, false>(st, a, n_sm);
+  if (a.count_work) return launch_trace_t<kP, true, kBatch, false, false>(st, a, n_sm);
+  if constexpr (!Prec<kP>::chain64)
+    if (a.group_log2 > 0) return launch_trace_t<kP, false, kBatch, false, true>(st, a, n_sm);
+  return launch_trace_t<kP, false, kBatch, false, false>(st, a, n_sm);
 }
 
 template <bool kBatch>
