@@ -211,7 +211,16 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   unsigned long long n_cand = 0, n_contrib = 0;
   const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long base = warp0 * 32; base < n_items; base += n_warps * 32) {
+  // Items a warp takes at a time: 32, one per lane, or fewer when that would
+  // leave warps without any -- a few segments can hold thousands of candidates,
+  // which a warp tests 32 at a time, so a small launch lasts as long as its
+  // fullest warp (17,700 segments with 28 candidates each on average: 617 ->
+  // 186 us).
+  int lg = 5;
+  while (lg > 0 && n_items < n_warps << lg) lg--;
+  const unsigned per = 1u << lg;
+  for (long long turn = warp0; turn << lg < n_items; turn += n_warps) {
+    const long long base = turn << lg;
     // ---- 1. one item per lane: segment parameters and the layer's footprint
     const long long it = base + lane;
     const long long ii = it / n_layers;
@@ -219,7 +228,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
     // the segment record: in order of place when the scene orders its scatter
     const long long si = a.order && it < n_items ? (long long)__ldg(&a.order[ii]) : ii;
     int nrows = 0;
-    if (it < n_items) {
+    if (lane < per && it < n_items) {
       // the footprint needs the apex, the cone normals and the start and end
       // planes (the record's first 112 bytes); the rest is read only for a
       // non-empty footprint
