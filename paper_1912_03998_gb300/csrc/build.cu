@@ -8,7 +8,7 @@
 // split, and a bottom-up pass that fills both child boxes of every node.
 //
 // Microphones (Section 3 partitions microphones together with the geometry):
-// keyed by their xy cell on a uniform grid, radix-sorted, and indexed by a
+// keyed by their cell on a uniform grid, sorted by counting, and indexed by a
 // cell-start table, so a row of cells is one contiguous run of microphones.
 #include <stdio.h>
 
@@ -31,19 +31,34 @@ __global__ void k_box_init(float *box) {
   else if (threadIdx.x < 6) box[threadIdx.x] = -kInf;
 }
 
-__device__ __forceinline__ void warp_box_reduce(float *lo, float *hi, float *box) {
+// Box of a block's threads into `box`, six atomics a block (they all go to the
+// same six words, so the callers keep the grid to kBoxBlocks: 787 blocks with
+// six atomics a warp spent 27 us on 201,381 triangles, most of it there).
+constexpr int kBoxThreads = 256, kBoxBlocks = 304;
+__device__ __forceinline__ void block_box_reduce(float *lo, float *hi, float *box) {
+  __shared__ float part[6][kBoxThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int k = 0; k < 3; k++) {
     for (int o = 16; o > 0; o >>= 1) {
       lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
       hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
     }
+    if (lane == 0) {
+      part[k][warp] = lo[k];
+      part[3 + k][warp] = hi[k];
+    }
   }
-  if ((threadIdx.x & 31) == 0) {
-    for (int k = 0; k < 3; k++) {
-      if (lo[k] <= hi[k]) {
-        atomic_min_f(&box[k], lo[k]);
-        atomic_max_f(&box[3 + k], hi[k]);
-      }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    const int k = threadIdx.x;
+    float l = part[k][0], h = part[3 + k][0];
+    for (int w = 1; w < kBoxThreads / 32; w++) {
+      l = fminf(l, part[k][w]);
+      h = fmaxf(h, part[3 + k][w]);
+    }
+    if (l <= h) {
+      atomic_min_f(&box[k], l);
+      atomic_max_f(&box[3 + k], h);
     }
   }
 }
@@ -51,7 +66,7 @@ __device__ __forceinline__ void warp_box_reduce(float *lo, float *hi, float *box
 // ------------------------------------------------------- triangle validation
 // Checks indices, materials and coordinates; accumulates the scene box over
 // valid triangles.  A bad triangle sets the error flag and is never read.
-__global__ void k_tri_validate(const float *verts, int64_t n_verts, const int32_t *tris,
+__global__ void __launch_bounds__(kBoxThreads) k_tri_validate(const float *verts, int64_t n_verts, const int32_t *tris,
                                int64_t n_tris, const uint8_t *mat, int n_mat, float *box, int *error) {
   float lo[3] = {kInf, kInf, kInf}, hi[3] = {-kInf, -kInf, -kInf};
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n_tris;
@@ -70,7 +85,7 @@ __global__ void k_tri_validate(const float *verts, int64_t n_verts, const int32_
       }
     }
   }
-  warp_box_reduce(lo, hi, box);
+  block_box_reduce(lo, hi, box);
 }
 
 // Spread the low 10 bits of v to every third bit.
@@ -137,14 +152,31 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint32_t *keys, in
   hist[threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
 }
 
-// In-place exclusive scan with one block of 1024 threads (sizes up to ~1e6).
+// In-place exclusive scan with one block of 1024 threads, 16 consecutive
+// entries each (one entry each took 24 us for the 25,344 digit counts of
+// 201,381 keys, a round trip to memory per 1,024 entries).
+constexpr int kScanPer = 16;
 __global__ void __launch_bounds__(1024) k_scan_excl(uint32_t *a, int n) {
   __shared__ uint32_t ws[32];
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t carry = 0;
-  for (int base = 0; base < n; base += 1024) {
-    int i = base + threadIdx.x;
-    uint32_t v = i < n ? a[i] : 0u, x = v;
+  for (int64_t base = 0; base < n; base += 1024 * kScanPer) {
+    const int64_t i0 = base + (int64_t)threadIdx.x * kScanPer;
+    uint32_t v[kScanPer], sum = 0;
+    const bool whole = i0 + kScanPer <= n;  // (16-byte aligned: the arrays are, and i0 is a multiple of 16)
+    if (whole) {
+#pragma unroll
+      for (int q = 0; q < kScanPer / 4; q++) {
+        const uint4 x = reinterpret_cast<const uint4 *>(a + i0)[q];
+        v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kScanPer; q++) v[q] = i0 + q < n ? a[i0 + q] : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < kScanPer; q++) sum += v[q];
+    uint32_t x = sum;
     for (int o = 1; o < 32; o <<= 1) {
       uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
@@ -160,9 +192,23 @@ __global__ void __launch_bounds__(1024) k_scan_excl(uint32_t *a, int n) {
       ws[lane] = s;
     }
     __syncthreads();
-    uint32_t incl = x + (warp > 0 ? ws[warp - 1] : 0u);
-    if (i < n) a[i] = carry + incl - v;
-    uint32_t total = ws[31];
+    uint32_t run = carry + x - sum + (warp > 0 ? ws[warp - 1] : 0u);
+#pragma unroll
+    for (int q = 0; q < kScanPer; q++) {
+      const uint32_t t = v[q];
+      v[q] = run;
+      run += t;
+    }
+    if (whole) {
+#pragma unroll
+      for (int q = 0; q < kScanPer / 4; q++)
+        reinterpret_cast<uint4 *>(a + i0)[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < kScanPer; q++)
+        if (i0 + q < n) a[i0 + q] = v[q];
+    }
+    const uint32_t total = ws[31];
     __syncthreads();
     carry += total;
   }
@@ -492,9 +538,8 @@ cudaError_t validate_scene(cudaStream_t st, const float *d_verts, int64_t n_vert
   k_box_init<<<1, 32, 0, st>>>(d_box);
   note_launches(1);
   if (n_tris == 0) return cudaGetLastError();
-  int threads = 256;
-  int64_t blocks = (n_tris + threads - 1) / threads;
-  k_tri_validate<<<(int)(blocks < 4096 ? blocks : 4096), threads, 0, st>>>(d_verts, n_verts, d_tris,
+  const int64_t blocks = (n_tris + kBoxThreads - 1) / kBoxThreads;
+  k_tri_validate<<<(int)(blocks < kBoxBlocks ? blocks : kBoxBlocks), kBoxThreads, 0, st>>>(d_verts, n_verts, d_tris,
                                                                           n_tris, d_mat, n_mat, d_box,
                                                                           d_error);
   note_launches(1);
@@ -712,7 +757,7 @@ cudaError_t tiled_build(cudaStream_t st, const Tri *src, const Plane *sp, const 
 }
 
 // ------------------------------------------------------------ microphones
-__global__ void k_mic_validate(const float *pos, int64_t n, float *box, int *error) {
+__global__ void __launch_bounds__(kBoxThreads) k_mic_validate(const float *pos, int64_t n, float *box, int *error) {
   float lo[3] = {kInf, kInf, kInf}, hi[3] = {-kInf, -kInf, -kInf};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -723,7 +768,7 @@ __global__ void k_mic_validate(const float *pos, int64_t n, float *box, int *err
       hi[k] = fmaxf(hi[k], c);
     }
   }
-  warp_box_reduce(lo, hi, box);
+  block_box_reduce(lo, hi, box);
 }
 
 __global__ void k_mic_grid(const float *box, int nx, int ny, int nz, int64_t n, MicGrid *g) {
@@ -748,44 +793,47 @@ __global__ void k_mic_grid(const float *box, int nx, int ny, int nz, int64_t n, 
   *g = r;
 }
 
-__global__ void k_mic_keys(const float *pos, int64_t n, const MicGrid *g, uint32_t *keys, uint32_t *vals) {
+// A counting sort by cell: each microphone's cell and its place among the
+// cell's microphones (any order serves: a microphone's result does not depend
+// on its place), the cells' starts by a scan, then the microphones to their
+// places -- three passes instead of the three per digit of a radix sort.
+// Microphones of a warp in the same cell take their places with one atomic.
+__global__ void k_mic_keys(const float *pos, int64_t n, const MicGrid *g, uint32_t *cell_count, uint2 *place) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  MicGrid gr = *g;
-  int cx = clampi((int)floorf((pos[3 * i] - gr.x0) * gr.inv_cw), 0, gr.nx - 1);
-  int cy = clampi((int)floorf((pos[3 * i + 1] - gr.y0) * gr.inv_ch), 0, gr.ny - 1);
-  int cz = gr.nz > 1 ? clampi((int)floorf((pos[3 * i + 2] - gr.z0) * gr.inv_dz), 0, gr.nz - 1) : 0;
-  keys[i] = (uint32_t)((cz * gr.ny + cy) * gr.nx + cx);
-  vals[i] = (uint32_t)i;
+  const bool ok = i < n;
+  uint32_t key = 0xffffffffu;
+  if (ok) {
+    MicGrid gr = *g;
+    int cx = clampi((int)floorf((pos[3 * i] - gr.x0) * gr.inv_cw), 0, gr.nx - 1);
+    int cy = clampi((int)floorf((pos[3 * i + 1] - gr.y0) * gr.inv_ch), 0, gr.ny - 1);
+    int cz = gr.nz > 1 ? clampi((int)floorf((pos[3 * i + 2] - gr.z0) * gr.inv_dz), 0, gr.nz - 1) : 0;
+    key = (uint32_t)((cz * gr.ny + cy) * gr.nx + cx);
+  }
+  const unsigned peers = __match_any_sync(0xffffffffu, key), lane = threadIdx.x & 31u;
+  const int leader = __ffs(peers) - 1;
+  uint32_t at = 0;
+  if (ok && (int)lane == leader) at = atomicAdd(&cell_count[key], (uint32_t)__popc(peers));
+  at = __shfl_sync(0xffffffffu, at, leader);
+  if (ok) place[i] = make_uint2(key, at + (uint32_t)__popc(peers & ((1u << lane) - 1u)));
 }
 
-__global__ void k_mic_gather(const float *pos, int64_t n, const uint32_t *keys, const uint32_t *vals,
-                             int n_cells, float4 *sorted, int *cell_start) {
+__global__ void k_mic_place(const float *pos, int64_t n, const int *cell_start, const uint2 *place, float4 *sorted) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  uint32_t v = vals[i];
-  sorted[i] = make_float4(pos[3 * (int64_t)v], pos[3 * (int64_t)v + 1], pos[3 * (int64_t)v + 2],
-                          __int_as_float((int)v));
-  int k = (int)keys[i];
-  int kp = i > 0 ? (int)keys[i - 1] : -1;
-  for (int c = kp + 1; c <= k; c++) cell_start[c] = (int)i;
-  if (i == n - 1)
-    for (int c = k + 1; c <= n_cells; c++) cell_start[c] = (int)n;
+  const uint2 p = place[i];
+  sorted[(uint32_t)cell_start[p.x] + p.y] =
+      make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __int_as_float((int)i));
 }
 
-size_t build_mics_scratch_bytes(int64_t n_m) {
-  size_t m = (size_t)(n_m > 0 ? n_m : 1);
-  return 4 * align256(4 * m) + align256(4 * rs_hist_entries((int)m));
-}
+size_t build_mics_scratch_bytes(int64_t n_m) { return align256(sizeof(uint2) * (size_t)(n_m > 0 ? n_m : 1)); }
 
 // The microphones' box (and a non-finite check); the host reads the box to
 // choose the grid before build_mics.
 cudaError_t mic_box(cudaStream_t st, const float *d_pos, int64_t n_m, float *d_box, int *d_error) {
   k_box_init<<<1, 32, 0, st>>>(d_box);
-  int threads = 256;
-  int64_t blocks = (n_m + threads - 1) / threads;
+  int64_t blocks = (n_m + kBoxThreads - 1) / kBoxThreads;
   if (blocks < 1) blocks = 1;
-  k_mic_validate<<<(int)(blocks < 4096 ? blocks : 4096), threads, 0, st>>>(d_pos, n_m, d_box, d_error);
+  k_mic_validate<<<(int)(blocks < kBoxBlocks ? blocks : kBoxBlocks), kBoxThreads, 0, st>>>(d_pos, n_m, d_box, d_error);
   note_launches(2);
   return cudaGetLastError();
 }
@@ -794,31 +842,18 @@ cudaError_t build_mics(cudaStream_t st, const float *d_pos, int64_t n_m, int nx,
                        const float *d_box, MicGrid *d_grid, float4 *d_sorted, int *d_cell_start, void *d_scratch,
                        size_t scratch_bytes) {
   if (scratch_bytes < build_mics_scratch_bytes(n_m)) return cudaErrorInvalidValue;
-  int n = (int)n_m;
-  size_t m = (size_t)(n > 0 ? n : 1);
-  char *s = (char *)d_scratch;
-  uint32_t *keys = (uint32_t *)s; s += align256(4 * m);
-  uint32_t *vals = (uint32_t *)s; s += align256(4 * m);
-  uint32_t *kalt = (uint32_t *)s; s += align256(4 * m);
-  uint32_t *valt = (uint32_t *)s; s += align256(4 * m);
-  uint32_t *hist = (uint32_t *)s;
+  uint2 *const place = (uint2 *)d_scratch;
   k_mic_grid<<<1, 1, 0, st>>>(d_box, nx, ny, nz, n_m, d_grid);
   note_launches(1);
   const int n_cells = nx * ny * nz;
-  if (n == 0) {
-    cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (n_cells + 1), st);
-    return cudaGetLastError();
-  }
-  int threads = 256;
-  int blocks = (n + threads - 1) / threads;
-  k_mic_keys<<<blocks, threads, 0, st>>>(d_pos, n_m, d_grid, keys, vals);
-  note_launches(1);
-  int bits = 1;
-  while ((1 << bits) < n_cells) bits++;
-  cudaError_t e = radix_sort(st, keys, vals, kalt, valt, hist, n, bits);
-  if (e != cudaSuccess) return e;
-  k_mic_gather<<<blocks, threads, 0, st>>>(d_pos, n_m, keys, vals, n_cells, d_sorted, d_cell_start);
-  note_launches(1);
+  // counts, and zero behind them: the scan leaves the starts and the total
+  cudaError_t e = cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (n_cells + 1), st);
+  if (e != cudaSuccess || n_m == 0) return e;
+  const int threads = 256, blocks = (int)((n_m + threads - 1) / threads);
+  k_mic_keys<<<blocks, threads, 0, st>>>(d_pos, n_m, d_grid, (uint32_t *)d_cell_start, place);
+  k_scan_excl<<<1, 1024, 0, st>>>((uint32_t *)d_cell_start, n_cells + 1);
+  k_mic_place<<<blocks, threads, 0, st>>>(d_pos, n_m, d_cell_start, place, d_sorted);
+  note_launches(3);
   return cudaGetLastError();
 }
 
