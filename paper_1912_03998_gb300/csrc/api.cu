@@ -89,8 +89,12 @@ struct SceneState {
 // several scenes can be in flight on the context's stream (bt_submit).
 struct TraceRec {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, done = nullptr;
-  std::vector<cudaEvent_t> kev;
-  std::vector<int> kind;  // kind of each pair of events in kev
+  std::vector<cudaEvent_t> kev;  // further events, reused by every trace
+  struct Span {
+    cudaEvent_t from, to;
+    int kind;
+  };
+  std::vector<Span> spans;  // each launch's events and kind; neighbours share theirs
   int64_t beams = 0, trace_launches = 0, scatter_launches = 0, rounds = 0;
 };
 
@@ -273,10 +277,11 @@ int collect(bt_ctx *c, int id, bool wait, bool report) {
   float ms = 0.0f;
   double trace_kms = 0.0, scatter_kms = 0.0;
   if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, r.ev0, r.ev1);
-  for (size_t q = 0; e == cudaSuccess && q + 1 < r.kev.size() && q / 2 < r.kind.size(); q += 2) {
+  for (const TraceRec::Span &q : r.spans) {
+    if (e != cudaSuccess) break;
     float a = 0.0f;
-    e = cudaEventElapsedTime(&a, r.kev[q], r.kev[q + 1]);
-    if (r.kind[q / 2] == 0) trace_kms += a;
+    e = cudaEventElapsedTime(&a, q.from, q.to);
+    if (q.kind == 0) trace_kms += a;
     else scatter_kms += a;
   }
   if (e != cudaSuccess) {
@@ -461,10 +466,12 @@ BT_API int bt_create(bt_ctx **out, int device, void *cuda_stream) {
       if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { rc = BT_E_CUDA; break; }
       c->own_stream = true;
     }
-    if (cudaMalloc(&c->d_ctr, sizeof(bt::Counters)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
-    if (cudaMalloc(&c->d_seg_count, sizeof(unsigned long long)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
+    // the counters and, right behind them, the two launch cursors, so that one
+    // clear covers all
+    if (cudaMalloc(&c->d_ctr, sizeof(bt::Counters) + 2 * sizeof(unsigned long long)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
+    c->d_seg_count = (unsigned long long *)(c->d_ctr + 1);
+    c->d_lineage_next = c->d_seg_count + 1;
     if (cudaMalloc(&c->d_box, 8 * sizeof(float)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
-    if (cudaMalloc(&c->d_lineage_next, sizeof(unsigned long long)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
     if (cudaMallocHost(&c->h_ctr, sizeof(bt::Counters)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
     if (cudaMallocHost(&c->h_sctr, sizeof(bt::Counters) * BT_MAX_SCENES) != cudaSuccess) { rc = BT_E_NOMEM; break; }
     if (cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess) { rc = BT_E_CUDA; break; }
@@ -501,9 +508,7 @@ BT_API int bt_destroy(bt_ctx *c) {
   release(c->order_hist);
   release(c->beam_table);
   if (c->d_ctr) cudaFree(c->d_ctr);
-  if (c->d_seg_count) cudaFree(c->d_seg_count);
   if (c->d_box) cudaFree(c->d_box);
-  if (c->d_lineage_next) cudaFree(c->d_lineage_next);
   if (c->h_ctr) cudaFreeHost(c->h_ctr);
   if (c->h_sctr) cudaFreeHost(c->h_sctr);
   for (TraceRec &r : c->rec) {
@@ -946,6 +951,8 @@ static void fill_view(bt::SceneView &v, SceneState &s, const bt_trace_params *p,
 // scatter by place.
 constexpr int64_t kOrderMics = (int64_t)1 << 20;
 
+constexpr int64_t kChunkFloor = (int64_t)1 << 30;  // bytes
+
 // Lineages per persistent launch when the caller leaves it to the library:
 // segment records of at most a quarter of the free device memory and at most
 // 32 GiB (fewer, larger launches have fewer launch tails), at least 1 GiB.
@@ -957,7 +964,7 @@ static int64_t default_chunk(int max_order) {
     if (budget > ((int64_t)32 << 30)) budget = (int64_t)32 << 30;
   }
   cudaGetLastError();
-  if (budget < ((int64_t)1 << 30)) budget = (int64_t)1 << 30;
+  if (budget < kChunkFloor) budget = kChunkFloor;
   return budget / ((int64_t)sizeof(bt::Seg) * (max_order + 1));
 }
 
@@ -965,7 +972,11 @@ static int64_t default_chunk(int max_order) {
 // the whole batch, and small enough that a launch's segment records are
 // indexed by int32 (the scatter keeps record indices in 32 bits).
 static int64_t launch_chunk(int32_t chunk_beams, int64_t total, int max_order) {
-  int64_t chunk = chunk_beams > 0 ? chunk_beams : default_chunk(max_order);
+  // (records that fit default_chunk's least budget need no look at the device's
+  // free memory, which costs a small trace more than its launches)
+  int64_t chunk = chunk_beams > 0 ? chunk_beams
+                  : total <= kChunkFloor / ((int64_t)sizeof(bt::Seg) * (max_order + 1)) ? total
+                                                                                        : default_chunk(max_order);
   const int64_t max_chunk = (int64_t)INT32_MAX / (max_order + 1);
   if (chunk > max_chunk) chunk = max_chunk;
   if (chunk > total) chunk = total;
@@ -1038,7 +1049,7 @@ static int enqueue_trace(bt_ctx *c, int32_t id, const bt_trace_params *p) {
   TraceRec &r = c->rec[id];
   for (cudaEvent_t *e : {&r.ev0, &r.ev1, &r.done})
     if (!*e) CK(cudaEventCreate(e));
-  r.kind.clear();
+  r.spans.clear();
   cudaStream_t st = c->stream;
   const int64_t n_beams = (int64_t)20 << (2 * s->level);
   const int64_t total = s->n_src * n_beams;
@@ -1076,9 +1087,8 @@ static int enqueue_trace(bt_ctx *c, int32_t id, const bt_trace_params *p) {
   } else {
     TRY(apply_leaf_size(c, *s, p, false));
   }
-  TRY(reset_counters(c));
-  CK(cudaMemsetAsync(s->energy.p, 0, sizeof(double) * bt::kMaxBands * (size_t)s->n_mics, st));
-  CK(cudaMemsetAsync(s->count.p, 0, sizeof(int) * (size_t)s->n_mics, st));
+  // accumulators, counters and cursors
+  CK(bt::launch_clear(st, (double *)s->energy.p, (int *)s->count.p, s->n_mics, c->d_ctr, c->d_seg_count, c->n_sm));
   bt::TraceArgs ta;
   memset(&ta, 0, sizeof(ta));
   fill_view(ta.v, *s, p, alpha_log2, has_alpha);
@@ -1142,54 +1152,58 @@ static int enqueue_trace(bt_ctx *c, int32_t id, const bt_trace_params *p) {
     tga.watchdog_ns = (unsigned long long)(p->watchdog_ms > 0 ? p->watchdog_ms : 2000) * 1000000ull;
     tga.withhold = p->fault_test == BT_FAULT_WITHHOLD ? 1 : 0;
   }
-  // Events bracket every launch: a pair per launch, its kind in r.kind.
+  // Events bracket every launch; the whole trace's first and last are its own.
   int n_ev = 0;
-  auto mark = [&](int kind) -> int {
-    while ((int)r.kev.size() < n_ev + 1) {
-      cudaEvent_t e;
-      CK(cudaEventCreate(&e));
-      r.kev.push_back(e);
+  cudaEvent_t at = nullptr;  // the event recorded last
+  auto mark = [&](cudaEvent_t ev) -> int {
+    if (!ev) {
+      if ((int)r.kev.size() < n_ev + 1) {
+        CK(cudaEventCreate(&ev));
+        r.kev.push_back(ev);
+      }
+      ev = r.kev[n_ev++];
     }
-    CK(cudaEventRecord(r.kev[n_ev], st));
-    if (n_ev % 2 == 0) r.kind.push_back(kind);
-    n_ev++;
+    CK(cudaEventRecord(ev, st));
+    at = ev;
     return BT_OK;
   };
-  auto scatter_round = [&]() -> int {
-    if (s->n_mics <= 0) return BT_OK;
-    TRY(mark(1));
-    if (by_place)
-      CK(bt::launch_seg_order(st, ta.segs, c->d_seg_count, ta.seg_capacity, ta.v.grid,
-                              (uint32_t *)c->order_hist.p, (uint32_t *)c->seg_order.p, c->n_sm));
-    CK(bt::launch_scatter(st, sa, c->n_sm));
-    return mark(1);
+  auto span = [&](int kind, cudaEvent_t end) -> int {
+    const cudaEvent_t from = at;
+    TRY(mark(end));
+    r.spans.push_back(TraceRec::Span{from, at, kind});
+    return BT_OK;
   };
   const int64_t n_chunks = total > 0 ? (total + chunk - 1) / chunk : 0;
   int64_t n_trace_launches = 0, n_scatter_launches = 0, n_rounds = 0;
-  CK(cudaEventRecord(r.ev0, st));
+  TRY(mark(r.ev0));
   for (int64_t ci = 0; ci < n_chunks; ci++) {
     int64_t b0 = ci * chunk;
+    const bool last = ci + 1 == n_chunks, scatters = s->n_mics > 0;
     ta.lineage_begin = b0;
     ta.lineage_end = b0 + chunk < total ? b0 + chunk : total;
-    CK(cudaMemsetAsync(c->d_seg_count, 0, sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(c->d_lineage_next, 0, sizeof(unsigned long long), st));
+    if (ci > 0) CK(cudaMemsetAsync(c->d_seg_count, 0, 2 * sizeof(unsigned long long), st));
     if (tiled) {
       CK(cudaMemsetAsync(c->t_seq.p, 0, sizeof(unsigned) * (size_t)T * qcap, st));
       CK(cudaMemsetAsync(c->t_qctl.p, 0, sizeof(int) * (3 * (size_t)T + 3), st));
     }
-    TRY(mark(0));
+    if (ci > 0 || tiled) TRY(mark(nullptr));
     if (tiled) {
       CK(bt::launch_trace_tiled(st, ta, tga, c->n_sm));
       n_rounds++;
     } else {
       CK(bt::launch_trace(st, ta, c->n_sm));
     }
-    TRY(mark(0));
+    TRY(span(0, last && !scatters ? r.ev1 : nullptr));
     n_trace_launches++;
-    TRY(scatter_round());
-    n_scatter_launches += s->n_mics > 0;
+    if (!scatters) continue;
+    if (by_place)
+      CK(bt::launch_seg_order(st, ta.segs, c->d_seg_count, ta.seg_capacity, ta.v.grid,
+                              (uint32_t *)c->order_hist.p, (uint32_t *)c->seg_order.p, c->n_sm));
+    CK(bt::launch_scatter(st, sa, c->n_sm));
+    TRY(span(1, last ? r.ev1 : nullptr));
+    n_scatter_launches++;
   }
-  CK(cudaEventRecord(r.ev1, st));
+  if (n_chunks == 0) TRY(mark(r.ev1));
   CK(cudaMemcpyAsync(&c->h_sctr[id], c->d_ctr, sizeof(bt::Counters), cudaMemcpyDeviceToHost, st));
   CK(cudaEventRecord(r.done, st));
   r.beams = total;
@@ -1267,17 +1281,38 @@ BT_API int bt_read_levels(bt_ctx *c, int32_t scene_id, double *level_db, double 
   }
   DeviceGuard g(c->device);
   cudaStream_t st = c->stream;
+  // device outputs are written in place, the others through the scene's
+  // read-back buffers
   const size_t nv = (size_t)s->n_mics * s->n_bands;
-  TRY(ensure(c, s->out_level, sizeof(double) * nv));
-  TRY(ensure(c, s->out_int, sizeof(double) * nv));
-  TRY(ensure(c, s->out_cnt, sizeof(int) * (size_t)s->n_mics));
+  auto direct = [&](const void *p, size_t align) { return p && (size_t)p % align == 0 && is_device_ptr(p, c->device); };
+  double *lv = nullptr, *in = nullptr;
+  int *ct = nullptr;
+  if (level_db && nv) {
+    lv = level_db;
+    if (!direct(level_db, sizeof(double))) {
+      TRY(ensure(c, s->out_level, sizeof(double) * nv));
+      lv = (double *)s->out_level.p;
+    }
+  }
+  if (intensity && nv) {
+    in = intensity;
+    if (!direct(intensity, sizeof(double))) {
+      TRY(ensure(c, s->out_int, sizeof(double) * nv));
+      in = (double *)s->out_int.p;
+    }
+  }
+  if (path_count && s->n_mics) {
+    ct = path_count;
+    if (!direct(path_count, sizeof(int))) {
+      TRY(ensure(c, s->out_cnt, sizeof(int) * (size_t)s->n_mics));
+      ct = (int *)s->out_cnt.p;
+    }
+  }
   CK(bt::launch_levels(st, (const double *)s->energy.p, (const int *)s->count.p, (const float4 *)s->mics.p,
-                       s->n_mics, s->n_bands, (double *)s->out_level.p, (double *)s->out_int.p,
-                       (int *)s->out_cnt.p));
-  if (level_db && nv) CK(cudaMemcpyAsync(level_db, s->out_level.p, sizeof(double) * nv, cudaMemcpyDefault, st));
-  if (intensity && nv) CK(cudaMemcpyAsync(intensity, s->out_int.p, sizeof(double) * nv, cudaMemcpyDefault, st));
-  if (path_count && s->n_mics)
-    CK(cudaMemcpyAsync(path_count, s->out_cnt.p, sizeof(int) * (size_t)s->n_mics, cudaMemcpyDefault, st));
+                       s->n_mics, s->n_bands, lv, in, ct));
+  if (lv && lv != level_db) CK(cudaMemcpyAsync(level_db, lv, sizeof(double) * nv, cudaMemcpyDefault, st));
+  if (in && in != intensity) CK(cudaMemcpyAsync(intensity, in, sizeof(double) * nv, cudaMemcpyDefault, st));
+  if (ct && ct != path_count) CK(cudaMemcpyAsync(path_count, ct, sizeof(int) * (size_t)s->n_mics, cudaMemcpyDefault, st));
   CK(cudaStreamSynchronize(st));
   if (stats) *stats = s->stats;
   return BT_OK;
@@ -1632,7 +1667,7 @@ BT_API int bt_trace_ranges(bt_ctx *c, int32_t n, const int32_t *scene_ids, const
   TRY(ensure(c, c->segs, sizeof(bt::Seg) * cap));
   TRY(ensure(c, c->views, sizeof(bt::SceneView) * (size_t)n));
   CK(cudaMemcpyAsync(c->views.p, hv.data(), sizeof(bt::SceneView) * (size_t)n, cudaMemcpyHostToDevice, st));
-  TRY(reset_counters(c));
+  CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(bt::Counters) + 2 * sizeof(unsigned long long), st));  // and the cursors
   for (int i = 0; i < n; i++) {
     SceneState &s = c->sc[scene_ids[i]];
     if (!(flags & BT_ACCUMULATE) && s.n_mics > 0) {
@@ -1682,8 +1717,7 @@ BT_API int bt_trace_ranges(bt_ctx *c, int32_t n, const int32_t *scene_ids, const
   for (int64_t ci = 0; ci < n_chunks; ci++) {
     ta.lineage_begin = first + ci * chunk;
     ta.lineage_end = ci * chunk + chunk < total ? ta.lineage_begin + chunk : first + total;
-    CK(cudaMemsetAsync(c->d_seg_count, 0, sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(c->d_lineage_next, 0, sizeof(unsigned long long), st));
+    if (ci > 0) CK(cudaMemsetAsync(c->d_seg_count, 0, 2 * sizeof(unsigned long long), st));
     CK(bt::launch_trace(st, ta, c->n_sm));
     CK(bt::launch_scatter(st, sa, c->n_sm));
   }
@@ -1772,18 +1806,6 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 // store the same address).
 std::atomic<void *> g_noalloc_ptr[256];
 
-__global__ void k_levels_noalloc(const double *energy, const int *count, const float4 *mics, int64_t n_m,
-                                 int n_bands, double *level_db, int *path_count) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n_m) return;
-  int64_t orig = __float_as_int(mics[p].w);
-  for (int b = 0; b < n_bands; b++) {
-    double I = energy[p * bt::kMaxBands + b];
-    level_db[orig * n_bands + b] = I > 0.0 ? 10.0 * log10(I) + 120.0 : -__builtin_huge_val();
-  }
-  if (path_count) path_count[orig] = count[p];
-}
-
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -1828,10 +1850,9 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
   const int mixed = p->precision == BT_PREC_MIXED ? 1 : 0;
   size_t off = 0;
   bt::Counters *ctr = (bt::Counters *)(base + off);
-  off = align_up(off + sizeof(bt::Counters), 256);
-  unsigned long long *seg_count = (unsigned long long *)(base + off);
+  unsigned long long *seg_count = (unsigned long long *)(ctr + 1);
   unsigned long long *lineage_next = seg_count + 1;
-  off = align_up(off + 2 * sizeof(unsigned long long), 256);
+  off = align_up(off + sizeof(bt::Counters) + 2 * sizeof(unsigned long long), 256);
   float *beam_table = (float *)(base + off);
   if (mixed) off = align_up(off + sizeof(float) * 24 * (size_t)n_beams, 256);
   bt::Seg *segs = (bt::Seg *)(base + off);
@@ -1843,9 +1864,7 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
   if (chunk > total) chunk = total > 0 ? total : 1;
   const unsigned long long cap = (unsigned long long)chunk * (p->max_order + 1);
   cudaStream_t st = c->stream;
-  CK(cudaMemsetAsync(ctr, 0, sizeof(bt::Counters), st));
-  CK(cudaMemsetAsync(s->energy.p, 0, sizeof(double) * bt::kMaxBands * (size_t)s->n_mics, st));
-  CK(cudaMemsetAsync(s->count.p, 0, sizeof(int) * (size_t)s->n_mics, st));
+  CK(bt::launch_clear(st, (double *)s->energy.p, (int *)s->count.p, s->n_mics, ctr, seg_count, c->n_sm));
   if (mixed && total > 0) CK(bt::launch_beam_table(st, s->level, beam_table));
   TRY(apply_leaf_size(c, *s, p, false));
   bt::TraceArgs ta;
@@ -1875,17 +1894,12 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
   for (int64_t ci = 0; ci < n_chunks; ci++) {
     ta.lineage_begin = ci * chunk;
     ta.lineage_end = ta.lineage_begin + chunk < total ? ta.lineage_begin + chunk : total;
-    CK(cudaMemsetAsync(seg_count, 0, 2 * sizeof(unsigned long long), st));
+    if (ci > 0) CK(cudaMemsetAsync(seg_count, 0, 2 * sizeof(unsigned long long), st));
     CK(bt::launch_trace(st, ta, c->n_sm));
     if (s->n_mics > 0) CK(bt::launch_scatter(st, sa, c->n_sm));
   }
-  if (s->n_mics > 0) {
-    k_levels_noalloc<<<(int)((s->n_mics + 255) / 256), 256, 0, st>>>(
-        (const double *)s->energy.p, (const int *)s->count.p, (const float4 *)s->mics.p, s->n_mics, s->n_bands,
-        level_db, path_count);
-    bt::note_launches(1);
-    CK(cudaGetLastError());
-  }
+  CK(bt::launch_levels(st, (const double *)s->energy.p, (const int *)s->count.p, (const float4 *)s->mics.p, s->n_mics,
+                       s->n_bands, level_db, nullptr, path_count));
   CK(cudaMemcpyAsync(c->h_ctr, ctr, sizeof(bt::Counters), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   const bt::Counters &h = *c->h_ctr;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "btrace.h"
 
 namespace bt {
@@ -556,6 +558,28 @@ __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? l
 
 // ------------------------------------------------------------ host launchers
 namespace bt {
+// A kernel's resident blocks per SM, asked of the runtime once per device (the
+// answer depends on nothing else; asking at every launch cost a small trace
+// several microseconds).  Host threads may ask at the same time.
+struct OccCache {
+  std::atomic<int> per_sm[64] = {};
+  template <typename K>
+  cudaError_t get(int *out, K kernel, int threads) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::atomic<int> *const slot = dev >= 0 && dev < 64 ? &per_sm[dev] : nullptr;
+    int v = slot ? slot->load(std::memory_order_relaxed) : 0;
+    if (v == 0) {
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, threads, 0);
+      if (e != cudaSuccess) return e;
+      if (v < 1) v = 1;
+      if (slot) slot->store(v, std::memory_order_relaxed);
+    }
+    *out = v;
+    return cudaSuccess;
+  }
+};
 // process-wide count of kernel launches (host side), read by bt_kernel_launches()
 void note_launches(int n);
 // scene build in two steps: validation (sets *d_error, fills the scene box)
@@ -602,6 +626,8 @@ constexpr int kOrderBits = 6, kOrderBins = 1 << (2 * kOrderBits);
 cudaError_t launch_seg_order(cudaStream_t st, const Seg *segs, const unsigned long long *seg_count,
                              unsigned long long cap, const MicGrid *grid, uint32_t *hist, uint32_t *order,
                              int n_sm);
+cudaError_t launch_clear(cudaStream_t st, double *energy, int *count, int64_t n_m, Counters *ctr,
+                         unsigned long long *cursors, int n_sm);
 cudaError_t launch_set_result(cudaStream_t st, const double *intensity, const int *count_in, const float4 *mics,
                               int64_t n_m, int n_bands, double *energy, int *count);
 // L2 read-bandwidth probe: `blocks` blocks of 256 threads read the n4 float4s

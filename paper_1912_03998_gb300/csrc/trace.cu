@@ -1827,9 +1827,9 @@ static int group_log2(int64_t n, int n_sm) {
 
 template <int kP, bool kCount, bool kLeaves, bool kGroup>
 static cudaError_t launch_tiled_t(cudaStream_t st, const TraceArgs &a, const TiledArgs &ta, int n_sm) {
+  static OccCache occ;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_tiled<kP, kCount, kLeaves, kGroup>,
-                                                                kTraceThreads, 0);
+  cudaError_t e = occ.get(&per_sm, k_trace_tiled<kP, kCount, kLeaves, kGroup>, kTraceThreads);
   if (e != cudaSuccess) return e;
   if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
   if (per_sm < 1) per_sm = 1;
@@ -1942,9 +1942,9 @@ cudaError_t launch_cast(cudaStream_t st, const DevScene &sc, const float *o, con
 // occupancy, each block looping until the batch's lineages are taken.
 template <int kP, bool kCount, bool kBatch, bool kLeaves, bool kGroup>
 static cudaError_t launch_trace_t(cudaStream_t st, const TraceArgs &a, int n_sm) {
+  static OccCache occ;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace<kP, kCount, kBatch, kLeaves, kGroup>,
-                                                                kTraceThreads, 0);
+  cudaError_t e = occ.get(&per_sm, k_trace<kP, kCount, kBatch, kLeaves, kGroup>, kTraceThreads);
   if (e != cudaSuccess) return e;
   if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_sm) per_sm = a.blocks_per_sm;
   if (per_sm < 1) per_sm = 1;
