@@ -466,9 +466,9 @@ BT_API int bt_create(bt_ctx **out, int device, void *cuda_stream) {
       if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { rc = BT_E_CUDA; break; }
       c->own_stream = true;
     }
-    // the counters and, right behind them, the two launch cursors, so that one
+    // the counters and, right behind them, the launch's cursors, so that one
     // clear covers all
-    if (cudaMalloc(&c->d_ctr, sizeof(bt::Counters) + 2 * sizeof(unsigned long long)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
+    if (cudaMalloc(&c->d_ctr, sizeof(bt::Counters) + bt::kCursors * sizeof(unsigned long long)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
     c->d_seg_count = (unsigned long long *)(c->d_ctr + 1);
     c->d_lineage_next = c->d_seg_count + 1;
     if (cudaMalloc(&c->d_box, 8 * sizeof(float)) != cudaSuccess) { rc = BT_E_NOMEM; break; }
@@ -1135,6 +1135,7 @@ static int enqueue_trace(bt_ctx *c, int32_t id, const bt_trace_params *p) {
   sa.max_nz = s->nz;
   sa.segs = ta.segs;
   sa.seg_count = c->d_seg_count;
+  sa.next = c->d_lineage_next + 1;
   sa.seg_capacity = ta.seg_capacity;
   sa.ctr = c->d_ctr;
   sa.order = by_place ? (const uint32_t *)c->seg_order.p : nullptr;
@@ -1181,7 +1182,7 @@ static int enqueue_trace(bt_ctx *c, int32_t id, const bt_trace_params *p) {
     const bool last = ci + 1 == n_chunks, scatters = s->n_mics > 0;
     ta.lineage_begin = b0;
     ta.lineage_end = b0 + chunk < total ? b0 + chunk : total;
-    if (ci > 0) CK(cudaMemsetAsync(c->d_seg_count, 0, 2 * sizeof(unsigned long long), st));
+    if (ci > 0) CK(cudaMemsetAsync(c->d_seg_count, 0, bt::kCursors * sizeof(unsigned long long), st));
     if (tiled) {
       CK(cudaMemsetAsync(c->t_seq.p, 0, sizeof(unsigned) * (size_t)T * qcap, st));
       CK(cudaMemsetAsync(c->t_qctl.p, 0, sizeof(int) * (3 * (size_t)T + 3), st));
@@ -1360,7 +1361,7 @@ struct bt_batch {
   int64_t total = 0, chunk = 1;
   DevBuf views, segs, beam_tables[9];
   bt::Counters *d_ctr = nullptr, *h_ctr = nullptr;
-  unsigned long long *d_cursors = nullptr;  // seg_count, lineage_next
+  unsigned long long *d_cursors = nullptr;  // kCursors
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   long long kernels_per_run = 0;
@@ -1450,7 +1451,7 @@ BT_API int bt_batch_create(bt_ctx *c, const int32_t *scene_ids, int32_t n_scenes
     if ((rc = ensure(c, b->segs, sizeof(bt::Seg) * (size_t)b->chunk * (b->max_order + 1)))) break;
     if (cudaMalloc(&b->d_ctr, sizeof(bt::Counters)) != cudaSuccess ||
         cudaMallocHost(&b->h_ctr, sizeof(bt::Counters)) != cudaSuccess ||
-        cudaMalloc(&b->d_cursors, 2 * sizeof(unsigned long long)) != cudaSuccess) {
+        cudaMalloc(&b->d_cursors, bt::kCursors * sizeof(unsigned long long)) != cudaSuccess) {
       rc = BT_E_NOMEM;
       break;
     }
@@ -1507,13 +1508,14 @@ static int record_batch(bt_batch *b) {
   sa.max_nz = b->max_nz;
   sa.segs = ta.segs;
   sa.seg_count = ta.seg_count;
+  sa.next = ta.lineage_next + 1;
   sa.seg_capacity = ta.seg_capacity;
   sa.ctr = b->d_ctr;
   const int64_t n_chunks = b->total > 0 ? (b->total + b->chunk - 1) / b->chunk : 0;
   for (int64_t ci = 0; ci < n_chunks; ci++) {
     ta.lineage_begin = ci * b->chunk;
     ta.lineage_end = ta.lineage_begin + b->chunk < b->total ? ta.lineage_begin + b->chunk : b->total;
-    CK(cudaMemsetAsync(b->d_cursors, 0, 2 * sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(b->d_cursors, 0, bt::kCursors * sizeof(unsigned long long), st));
     CK(bt::launch_trace(st, ta, c->n_sm));
     CK(bt::launch_scatter(st, sa, c->n_sm));
   }
@@ -1667,7 +1669,7 @@ BT_API int bt_trace_ranges(bt_ctx *c, int32_t n, const int32_t *scene_ids, const
   TRY(ensure(c, c->segs, sizeof(bt::Seg) * cap));
   TRY(ensure(c, c->views, sizeof(bt::SceneView) * (size_t)n));
   CK(cudaMemcpyAsync(c->views.p, hv.data(), sizeof(bt::SceneView) * (size_t)n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(bt::Counters) + 2 * sizeof(unsigned long long), st));  // and the cursors
+  CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(bt::Counters) + bt::kCursors * sizeof(unsigned long long), st));  // and the cursors
   for (int i = 0; i < n; i++) {
     SceneState &s = c->sc[scene_ids[i]];
     if (!(flags & BT_ACCUMULATE) && s.n_mics > 0) {
@@ -1710,6 +1712,7 @@ BT_API int bt_trace_ranges(bt_ctx *c, int32_t n, const int32_t *scene_ids, const
   sa.max_nz = max_nz;
   sa.segs = ta.segs;
   sa.seg_count = ta.seg_count;
+  sa.next = ta.lineage_next + 1;
   sa.seg_capacity = cap;
   sa.ctr = c->d_ctr;
   CK(cudaEventRecord(c->ev0, st));
@@ -1717,7 +1720,7 @@ BT_API int bt_trace_ranges(bt_ctx *c, int32_t n, const int32_t *scene_ids, const
   for (int64_t ci = 0; ci < n_chunks; ci++) {
     ta.lineage_begin = first + ci * chunk;
     ta.lineage_end = ci * chunk + chunk < total ? ta.lineage_begin + chunk : first + total;
-    if (ci > 0) CK(cudaMemsetAsync(c->d_seg_count, 0, 2 * sizeof(unsigned long long), st));
+    if (ci > 0) CK(cudaMemsetAsync(c->d_seg_count, 0, bt::kCursors * sizeof(unsigned long long), st));
     CK(bt::launch_trace(st, ta, c->n_sm));
     CK(bt::launch_scatter(st, sa, c->n_sm));
   }
@@ -1845,14 +1848,14 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
     g_noalloc_ptr[c->device].store(ptr, std::memory_order_release);
     base = (char *)ptr;
   }
-  // carve the scratch: counters, two cursors, beam table, segment records
+  // carve the scratch: counters, cursors, beam table, segment records
   const int64_t n_beams = (int64_t)20 << (2 * s->level);
   const int mixed = p->precision == BT_PREC_MIXED ? 1 : 0;
   size_t off = 0;
   bt::Counters *ctr = (bt::Counters *)(base + off);
   unsigned long long *seg_count = (unsigned long long *)(ctr + 1);
   unsigned long long *lineage_next = seg_count + 1;
-  off = align_up(off + sizeof(bt::Counters) + 2 * sizeof(unsigned long long), 256);
+  off = align_up(off + sizeof(bt::Counters) + bt::kCursors * sizeof(unsigned long long), 256);
   float *beam_table = (float *)(base + off);
   if (mixed) off = align_up(off + sizeof(float) * 24 * (size_t)n_beams, 256);
   bt::Seg *segs = (bt::Seg *)(base + off);
@@ -1888,13 +1891,14 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
   sa.max_nz = s->nz;
   sa.segs = segs;
   sa.seg_count = seg_count;
+  sa.next = lineage_next + 1;
   sa.seg_capacity = cap;
   sa.ctr = ctr;
   const int64_t n_chunks = total > 0 ? (total + chunk - 1) / chunk : 0;
   for (int64_t ci = 0; ci < n_chunks; ci++) {
     ta.lineage_begin = ci * chunk;
     ta.lineage_end = ta.lineage_begin + chunk < total ? ta.lineage_begin + chunk : total;
-    if (ci > 0) CK(cudaMemsetAsync(seg_count, 0, 2 * sizeof(unsigned long long), st));
+    if (ci > 0) CK(cudaMemsetAsync(seg_count, 0, bt::kCursors * sizeof(unsigned long long), st));
     CK(bt::launch_trace(st, ta, c->n_sm));
     if (s->n_mics > 0) CK(bt::launch_scatter(st, sa, c->n_sm));
   }

@@ -236,7 +236,11 @@ struct ScatterArgs {
   unsigned long long seg_capacity;
   Counters *ctr;
   const uint32_t *order;    // the emitted segments in order of place (launch_seg_order), or null
+  unsigned long long *next; // items taken so far (zero at launch)
 };
+// A launch's cursors, zero at its start: segments emitted, lineages taken,
+// scatter items taken.
+constexpr int kCursors = 3;
 
 // ------------------------------------------------------------------ helpers
 __device__ __forceinline__ float3 f3(float4 v) { return make_float3(v.x, v.y, v.z); }

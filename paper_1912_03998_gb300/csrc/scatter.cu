@@ -209,18 +209,29 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   const int n_layers = a.max_nz > 1 ? a.max_nz : 1;
   const long long n_items = n_seg * n_layers;
   unsigned long long n_cand = 0, n_contrib = 0;
-  const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-  // Items a warp takes at a time: 32, one per lane, or fewer when that would
-  // leave warps without any -- a few segments can hold thousands of candidates,
-  // which a warp tests 32 at a time, so a small launch lasts as long as its
-  // fullest warp (17,700 segments with 28 candidates each on average: 617 ->
-  // 186 us).
-  int lg = 5;
-  while (lg > 0 && n_items < n_warps << lg) lg--;
-  const unsigned per = 1u << lg;
-  for (long long turn = warp0; turn << lg < n_items; turn += n_warps) {
-    const long long base = turn << lg;
+  // Items a warp takes at a time: 32, one per lane, and fewer once less than
+  // that is left for every warp.  The first take is the warp's own, the
+  // others come from the launch's counter.  Segments differ by orders of
+  // magnitude -- a wide beam over open ground holds thousands of candidates,
+  // which a warp tests 32 at a time -- so with fixed shares a launch lasted as
+  // long as its fullest warp (eight uneven cities, 4.4 M segments: batch call
+  // 5.0 -> 4.3 ms; 17,700 segments of 28 candidates each on average: 617 -> 121
+  // us).  The
+  // next take is under way while a warp works.
+  auto share = [&](long long left) {
+    int lg = 5;
+    while (lg > 0 && left < n_warps << lg) lg--;
+    return lg;
+  };
+  const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  int lg = share(n_items);
+  const long long own = n_warps << lg;  // items of the first takes
+  unsigned long long taken = 0;
+  for (long long base = warp0 << lg; base < n_items;) {
+    const unsigned per = 1u << lg;
+    const int lg_next = share(n_items - max(base, own));
+    if (lane == 0 && own < n_items) taken = own + atomicAdd(a.next, 1ull << lg_next);
     // ---- 1. one item per lane: segment parameters and the layer's footprint
     const long long it = base + lane;
     const long long ii = it / n_layers;
@@ -468,6 +479,9 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
       }
     }
     __syncwarp();
+    if (own >= n_items) break;
+    base = (long long)__shfl_sync(0xffffffffu, taken, 0);
+    lg = lg_next;
   }
   for (int o = 16; o > 0; o >>= 1) {
     n_cand += __shfl_xor_sync(0xffffffffu, n_cand, o);
@@ -776,7 +790,7 @@ cudaError_t launch_levels(cudaStream_t st, const double *energy, const int *coun
   return cudaGetLastError();
 }
 
-// Clear a scene's accumulators and a trace's counters and two cursors, in one
+// Clear a scene's accumulators and a trace's counters and cursors, in one
 // launch instead of five (which took longer than a small trace's scatter).
 __global__ void __launch_bounds__(256) k_clear(double2 *energy, int *count, int64_t n_m, Counters *ctr,
                                                unsigned long long *cursors) {
@@ -785,7 +799,7 @@ __global__ void __launch_bounds__(256) k_clear(double2 *energy, int *count, int6
   for (int64_t i = i0; i < n_m * (kMaxBands / 2); i += step) energy[i] = make_double2(0.0, 0.0);
   for (int64_t i = i0; i < n_m; i += step) count[i] = 0;
   if (i0 < (int64_t)(sizeof(Counters) / 8)) ((unsigned long long *)ctr)[i0] = 0ull;
-  if (i0 < 2) cursors[i0] = 0ull;
+  if (i0 < kCursors) cursors[i0] = 0ull;
 }
 
 cudaError_t launch_clear(cudaStream_t st, double *energy, int *count, int64_t n_m, Counters *ctr,
