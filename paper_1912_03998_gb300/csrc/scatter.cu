@@ -205,9 +205,13 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   float(*F)[32] = sm.f[w];
   const long long n_seg = (long long)min(*a.seg_count, a.seg_capacity);
   // work items: (segment, microphone layer) pairs; one per segment when the
-  // microphones lie in one layer
+  // microphones lie in one layer.  By groups of 32 segments, layer by layer: a
+  // warp then takes one layer of 32 neighbours and not the 32 layers of one
+  // segment, which for a long beam over the roofs hold tens of thousands of
+  // candidates (13.75 M microphones, 8 sources: 40 % of the chip's time went
+  // by waiting for such warps; 10.1 -> 5.9 ms, 40 sources 29.9 -> 24.6 ms).
   const int n_layers = a.max_nz > 1 ? a.max_nz : 1;
-  const long long n_items = n_seg * n_layers;
+  const long long n_items = n_layers > 1 ? (n_seg + 31) / 32 * 32 * n_layers : n_seg;
   unsigned long long n_cand = 0, n_contrib = 0;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
   // Items a warp takes at a time: 32, one per lane, and fewer once less than
@@ -234,12 +238,18 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
     if (lane == 0 && own < n_items) taken = own + atomicAdd(a.next, 1ull << lg_next);
     // ---- 1. one item per lane: segment parameters and the layer's footprint
     const long long it = base + lane;
-    const long long ii = it / n_layers;
-    const int layer = (int)(it - ii * n_layers);
+    long long ii = it;
+    int layer = 0;
+    if (n_layers > 1) {
+      const long long group = it / (32 * n_layers);
+      const int rest = (int)(it - group * (32 * n_layers));
+      layer = rest >> 5;
+      ii = group * 32 + (rest & 31);
+    }
     // the segment record: in order of place when the scene orders its scatter
-    const long long si = a.order && it < n_items ? (long long)__ldg(&a.order[ii]) : ii;
+    const long long si = a.order && ii < n_seg ? (long long)__ldg(&a.order[ii]) : ii;
     int nrows = 0;
-    if (lane < per && it < n_items) {
+    if (lane < per && ii < n_seg) {
       // the footprint needs the apex, the cone normals and the start and end
       // planes (the record's first 112 bytes); the rest is read only for a
       // non-empty footprint
