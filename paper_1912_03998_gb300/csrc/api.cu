@@ -111,8 +111,8 @@ struct bt_ctx {
   char err[512] = {0};
   DevBuf scratch, stage_a, stage_b, stage_c, segs;
   DevBuf seg_order, order_hist;  // scatter in order of place (scenes with many microphones)
-  DevBuf beam_table;       // cone normals + axis per beam of one icosahedron level, float pairs
-  int beam_table_level = -1;
+  DevBuf beam_table[2];    // cone normals + axis per beam of one icosahedron level: float pairs, float64
+  int beam_table_level[2] = {-1, -1};
   bt::Counters *d_ctr = nullptr;
   bt::Counters *h_ctr = nullptr;  // pinned
   bt::Counters *h_sctr = nullptr; // pinned, one per scene slot: counters of the slot's last trace
@@ -126,7 +126,7 @@ struct bt_ctx {
   unsigned long long gen_counter = 0;
   std::vector<bt_batch *> batches;  // live batches, freed with the context
   DevBuf views;                     // scene views of the last bt_trace_ranges
-  DevBuf level_tables[9];           // float-pair beam tables per icosahedron level (bt_trace_ranges)
+  DevBuf level_tables[2][9];        // beam tables (float pairs, float64) per icosahedron level (bt_trace_ranges)
   bt_stats range_stats;             // totals of the last bt_trace_ranges
 };
 
@@ -495,7 +495,8 @@ BT_API int bt_destroy(bt_ctx *c) {
   for (bt_batch *b : c->batches) free_batch(b);
   c->batches.clear();
   release(c->views);
-  for (DevBuf &t : c->level_tables) release(t);
+  for (auto &k : c->level_tables)
+    for (DevBuf &t : k) release(t);
   for (auto &s : c->sc) release_scene(c, s);
   for (DevBuf &q : c->pool) release(q);
   c->pool.clear();
@@ -506,7 +507,7 @@ BT_API int bt_destroy(bt_ctx *c) {
   release(c->segs);
   release(c->seg_order);
   release(c->order_hist);
-  release(c->beam_table);
+  for (DevBuf &t : c->beam_table) release(t);
   if (c->d_ctr) cudaFree(c->d_ctr);
   if (c->d_box) cudaFree(c->d_box);
   if (c->h_ctr) cudaFreeHost(c->h_ctr);
@@ -1120,13 +1121,16 @@ static int enqueue_trace(bt_ctx *c, int32_t id, const bt_trace_params *p) {
     ta.hit_log = s->hit_log;
     ta.hit_log_stride = p->max_order + 1;
   }
-  if (ta.prec == BT_PREC_MIXED && total > 0) {
-    if (c->beam_table_level != s->level) {
-      TRY(ensure(c, c->beam_table, sizeof(float) * 24 * (size_t)n_beams));
-      CK(bt::launch_beam_table(st, s->level, (float *)c->beam_table.p));
-      c->beam_table_level = s->level;
+  if (ta.prec != BT_PREC_FP32 && total > 0) {
+    const int kind = ta.prec == BT_PREC_MIXED ? 0 : 1;
+    DevBuf &table = c->beam_table[kind];
+    if (c->beam_table_level[kind] != s->level) {
+      c->beam_table_level[kind] = -1;
+      TRY(ensure(c, table, bt::kBeamBytes * (size_t)n_beams));
+      CK(bt::launch_beam_table(st, ta.prec, s->level, (float *)table.p));
+      c->beam_table_level[kind] = s->level;
     }
-    ta.v.beam_table = (const float *)c->beam_table.p;
+    ta.v.beam_table = (const float *)table.p;
   }
   bt::ScatterArgs sa;
   memset(&sa, 0, sizeof(sa));
@@ -1436,11 +1440,11 @@ BT_API int bt_batch_create(bt_ctx *c, const int32_t *scene_ids, int32_t n_scenes
       b->total += s.n_src * nb;
       if (params[i].max_order > b->max_order) b->max_order = params[i].max_order;
       if (s.nz > b->max_nz) b->max_nz = s.nz;
-      if (prec == BT_PREC_MIXED && s.n_src > 0) {
+      if (prec != BT_PREC_FP32 && s.n_src > 0) {
         DevBuf &t = b->beam_tables[s.level];
         if (!t.p) {
-          if ((rc = ensure(c, t, sizeof(float) * 24 * (size_t)nb))) break;
-          if (bt::launch_beam_table(st, s.level, (float *)t.p) != cudaSuccess) { rc = BT_E_CUDA; break; }
+          if ((rc = ensure(c, t, bt::kBeamBytes * (size_t)nb))) break;
+          if (bt::launch_beam_table(st, prec, s.level, (float *)t.p) != cudaSuccess) { rc = BT_E_CUDA; break; }
         }
         hv[i].beam_table = (const float *)t.p;
       }
@@ -1655,11 +1659,11 @@ BT_API int bt_trace_ranges(bt_ctx *c, int32_t n, const int32_t *scene_ids, const
     total += lineage_end[i] - lineage_begin[i];
     if (p->max_order > kmax) kmax = p->max_order;
     if (s->nz > max_nz) max_nz = s->nz;
-    if (prec == BT_PREC_MIXED && nl > 0) {
-      DevBuf &t = c->level_tables[s->level];
+    if (prec != BT_PREC_FP32 && nl > 0) {
+      DevBuf &t = c->level_tables[prec == BT_PREC_MIXED ? 0 : 1][s->level];
       if (!t.p) {
-        TRY(ensure(c, t, sizeof(float) * 24 * (size_t)((int64_t)20 << (2 * s->level))));
-        CK(bt::launch_beam_table(st, s->level, (float *)t.p));
+        TRY(ensure(c, t, bt::kBeamBytes * (size_t)((int64_t)20 << (2 * s->level))));
+        CK(bt::launch_beam_table(st, prec, s->level, (float *)t.p));
       }
       hv[i].beam_table = (const float *)t.p;
     }
@@ -1850,14 +1854,14 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
   }
   // carve the scratch: counters, cursors, beam table, segment records
   const int64_t n_beams = (int64_t)20 << (2 * s->level);
-  const int mixed = p->precision == BT_PREC_MIXED ? 1 : 0;
+  const bool table = p->precision != BT_PREC_FP32;
   size_t off = 0;
   bt::Counters *ctr = (bt::Counters *)(base + off);
   unsigned long long *seg_count = (unsigned long long *)(ctr + 1);
   unsigned long long *lineage_next = seg_count + 1;
   off = align_up(off + sizeof(bt::Counters) + bt::kCursors * sizeof(unsigned long long), 256);
   float *beam_table = (float *)(base + off);
-  if (mixed) off = align_up(off + sizeof(float) * 24 * (size_t)n_beams, 256);
+  if (table) off = align_up(off + bt::kBeamBytes * (size_t)n_beams, 256);
   bt::Seg *segs = (bt::Seg *)(base + off);
   const unsigned long long seg_room = (kNoAllocBytes - off) / sizeof(bt::Seg);
   const int64_t total = s->n_src * n_beams;
@@ -1868,12 +1872,12 @@ BT_API int bt_trace_noalloc(bt_ctx *c, int32_t scene_id, const bt_trace_params *
   const unsigned long long cap = (unsigned long long)chunk * (p->max_order + 1);
   cudaStream_t st = c->stream;
   CK(bt::launch_clear(st, (double *)s->energy.p, (int *)s->count.p, s->n_mics, ctr, seg_count, c->n_sm));
-  if (mixed && total > 0) CK(bt::launch_beam_table(st, s->level, beam_table));
+  if (table && total > 0) CK(bt::launch_beam_table(st, p->precision, s->level, beam_table));
   TRY(apply_leaf_size(c, *s, p, false));
   bt::TraceArgs ta;
   memset(&ta, 0, sizeof(ta));
   fill_view(ta.v, *s, p, alpha_log2, has_alpha);
-  ta.v.beam_table = mixed ? beam_table : nullptr;
+  ta.v.beam_table = table ? beam_table : nullptr;
   ta.segs = segs;
   ta.seg_count = seg_count;
   ta.seg_capacity = cap;

@@ -196,7 +196,8 @@ struct SceneView {
   int has_alpha;
   int seg_key;            // 1: each segment record carries its grid cell (Seg::key)
   const MicGrid *grid;
-  const float *beam_table;   // MIXED: per beam 3 cone normals + axis as float pairs: [n_beams][12] hi, then lo
+  const float *beam_table;   // per beam 3 cone normals + axis: MIXED float pairs ([n_beams][12] hi, then lo), FP64
+                             // and MIXED64 [n_beams][12] doubles, FP32 none
   const float4 *mics;        // sorted by cell: xyz, w = original index (int bits)
   const int *cell_start;     // [nx * ny + 1]
   double *energy;            // [n_mics][kMaxBands], sorted order
@@ -595,7 +596,9 @@ cudaError_t build_scene(cudaStream_t st, const float *d_verts, const int32_t *d_
                         const uint8_t *d_mat, void *d_hier, Tri *d_tris_out, Plane *d_planes,
                         Plane64 *d_planes64, PlaneDF *d_planes_df, void *d_scratch, size_t scratch_bytes,
                         const float *d_box, int *d_error);
-cudaError_t launch_beam_table(cudaStream_t st, int level, float *table);
+// The beams of a level for a precision other than FP32, kBeamBytes a beam.
+constexpr size_t kBeamBytes = 96;
+cudaError_t launch_beam_table(cudaStream_t st, int prec, int level, float *table);
 cudaError_t launch_beam_axes(cudaStream_t st, int level, float *axes);
 size_t build_tiled_scratch_bytes(int64_t n_src, int64_t n_pairs);
 cudaError_t tiled_count(cudaStream_t st, const Tri *src, int64_t n_src, const TileGrid &tg, uint32_t *offs);

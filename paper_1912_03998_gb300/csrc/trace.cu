@@ -132,9 +132,29 @@ __global__ void k_beam_table(int level, int64_t n_beams, float *table) {
   }
 }
 
-cudaError_t launch_beam_table(cudaStream_t st, int level, float *table) {
+// The same in float64 for the float64-chain variants, 12 doubles a beam.  Those
+// formed each lineage's beam in the trace kernel: some thousand float64
+// operations for the few lanes of a service phase that start a lineage, which
+// cost as much of the float64 pipe as everything else together (FP64, 24
+// district sources: trace kernel 3.23 -> 2.31 ms).
+__global__ void k_beam_table64(int level, int64_t n_beams, double *table) {
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n_beams) return;
+  double3 d0, d1, d2;
+  beam_dirs<double>(level, i, d0, d1, d2);
+  const double3 v[4] = {cross_exact(d0, d1), cross_exact(d1, d2), cross_exact(d2, d0), normalize3((d0 + d1) + d2)};
+  double *o = table + 12 * i;
+  for (int k = 0; k < 4; k++) {
+    o[3 * k] = v[k].x;
+    o[3 * k + 1] = v[k].y;
+    o[3 * k + 2] = v[k].z;
+  }
+}
+
+cudaError_t launch_beam_table(cudaStream_t st, int prec, int level, float *table) {
   int64_t n = (int64_t)20 << (2 * level);
-  k_beam_table<<<(int)((n + 127) / 128), 128, 0, st>>>(level, n, table);
+  if (prec == kPMixed) k_beam_table<<<(int)((n + 127) / 128), 128, 0, st>>>(level, n, table);
+  else k_beam_table64<<<(int)((n + 127) / 128), 128, 0, st>>>(level, n, (double *)table);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -882,12 +902,17 @@ __device__ __forceinline__ void init_lineage(const SceneView &a, LineageSmem<kP,
   float4 s4 = __ldg(&a.src[si]);
   float3 A = make_float3(s4.x, s4.y, s4.z);
   if (kChain64) {
-    double3 d0, d1, d2;
-    beam_dirs<double>(a.level, bi, d0, d1, d2);
-    st_d3(sm, kRowN, t, cross_exact(d0, d1));
-    st_d3(sm, kRowN + 3, t, cross_exact(d1, d2));
-    st_d3(sm, kRowN + 6, t, cross_exact(d2, d0));
-    st_d3(sm, kRowD, t, normalize3((d0 + d1) + d2));
+    const double2 *bt = reinterpret_cast<const double2 *>(a.beam_table) + 6 * bi;
+    double d[12];
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+      const double2 x = __ldg(bt + q);
+      d[2 * q] = x.x;
+      d[2 * q + 1] = x.y;
+    }
+#pragma unroll
+    for (int j = 0; j < 3; j++) st_d3(sm, kRowN + 3 * j, t, make_double3(d[3 * j], d[3 * j + 1], d[3 * j + 2]));
+    st_d3(sm, kRowD, t, make_double3(d[9], d[10], d[11]));
     const double3 A64 = make_double3(s4.x, s4.y, s4.z);
     st_d3(sm, kRowA, t, A64);
     st_d3(sm, kRowO, t, A64);
