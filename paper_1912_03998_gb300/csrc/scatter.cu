@@ -192,6 +192,56 @@ __device__ __forceinline__ double plane_side64(const SceneView &a, int slot, flo
   return pl.x * nf.x + pl.y * nf.y + pl.z * nf.z < 0.0 ? -e : e;
 }
 
+// FP64: test microphone e.x against segment record e.y and add its
+// contribution, all in float64 (apex exact from its three words, cone normals
+// from their float pairs, start and end planes from the triangles' float64
+// planes).  1 if it contributed.
+template <bool kBatch>
+__device__ __forceinline__ int contribute64(const ScatterArgs &a, int2 e) {
+  const Seg *const rec = a.segs + e.y;
+  const SceneView &V = kBatch ? a.views[rec->view] : a.v;
+  const float4 m = __ldg(&V.mics[e.x]);
+  const float4 n0 = __ldg(&rec->n0), n1 = __ldg(&rec->n1), n2 = __ldg(&rec->n2);
+  const float4 st = __ldg(&rec->start), en = __ldg(&rec->end);
+  double3 vd;
+  vd.x = (double)m.x - (((double)__ldg(&rec->ahi[0]) + __ldg(&rec->alo[0])) + __ldg(&rec->pad[0]));
+  vd.y = (double)m.y - (((double)__ldg(&rec->ahi[1]) + __ldg(&rec->alo[1])) + __ldg(&rec->pad[1]));
+  vd.z = (double)m.z - (((double)__ldg(&rec->ahi[2]) + __ldg(&rec->alo[2])) + __ldg(&rec->pad[2]));
+  const float3 nh[3] = {f3(n0), f3(n1), f3(n2)};
+  bool in = true;
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    const double3 nd = make_double3((double)nh[j].x + __ldg(&rec->nlo[3 * j]), (double)nh[j].y + __ldg(&rec->nlo[3 * j + 1]),
+                                    (double)nh[j].z + __ldg(&rec->nlo[3 * j + 2]));
+    in = in && dot3(nd, vd) >= 0.0;
+  }
+  if (in) {
+    const int s_slot = __float_as_int(n0.w), e_slot = __float_as_int(n1.w);
+    const double fs = s_slot >= 0 ? plane_side64(V, s_slot, f3(st), m) : 1.0;
+    const double fe = e_slot >= 0 ? plane_side64(V, e_slot, f3(en), m) : 1.0;
+    in = fs > 0.0 && fe >= 0.0;
+  }
+  const double d2 = dot3(vd, vd);
+  if (!(in && d2 > 1e-18)) return 0;
+  const double gf = 1.0 / (4.0 * 3.141592653589793 * d2);
+  const bool has_alpha = V.has_alpha != 0;
+  const double dist = has_alpha ? sqrt(d2) : 0.0;
+  const float4 p0 = __ldg(&rec->p03), p1 = __ldg(&rec->p47);
+  const float p[kMaxBands] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+  double *const out = V.energy + (size_t)e.x * kMaxBands;
+  const int nb = V.sc.n_bands;
+#pragma unroll
+  for (int b = 0; b < kMaxBands; b++) {
+    if (b < nb) {
+      double c = (double)p[b] * gf;
+      if (has_alpha) c *= exp2((double)V.alpha_log2[b] * dist);
+      atomicAdd(out + b, c);
+    }
+  }
+  atomicAdd(V.count + e.x, 1);
+  return 1;
+}
+
 // One warp takes 32 segments at a time.  Each lane loads one segment and
 // builds its footprint; the warp then walks the (segment, cell row) pairs of
 // all 32 footprints 32 at a time, turns each into its run of microphones, and
@@ -213,6 +263,13 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   const int n_layers = a.max_nz > 1 ? a.max_nz : 1;
   const long long n_items = n_layers > 1 ? (n_seg + 31) / 32 * 32 * n_layers : n_seg;
   unsigned long long n_cand = 0, n_contrib = 0;
+  // FP64: candidates that wait for their float64 test, (microphone, segment),
+  // tested 32 at a time: whole-warp float64 instructions cost the same for one
+  // lane as for 32, and one candidate in ten comes this far (24 district
+  // sources: 1.07 -> 0.32 ms)
+  __shared__ int2 wait_q[kF64 ? kScatterWarps : 1][kF64 ? 64 : 1];
+  int2 *const wait = wait_q[kF64 ? w : 0];
+  int n_wait = 0;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
   // Items a warp takes at a time: 32, one per lane, and fewer once less than
   // that is left for every warp.  The first take is the warp's own, the
@@ -360,6 +417,8 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
         int ofirst = __shfl_sync(0xffffffffu, first, ro);
         int oexcl = __shfl_sync(0xffffffffu, cexcl, ro);
         int s = __shfl_sync(0xffffffffu, so, ro);
+        [[maybe_unused]] bool near = false;
+        [[maybe_unused]] int2 entry = make_int2(0, 0);
         if (c < total_c) {
           int mi = ofirst + (c - oexcl);
           // where the contribution goes: the scene's accumulators, band
@@ -386,55 +445,26 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
           }
           const Seg *rec = a.segs + __float_as_int(F[F_SI][s]);
           float4 m = __ldg(&mics[mi]);
-          if (kF64) {
-            // FP64: every test and the contribution in float64 (apex exact
-            // from its three words, cone normals from their float pairs,
-            // start/end planes from the triangles' float64 planes)
-            n_cand++;
-            const double3 A = make_double3(((double)F[F_AX][s] + F[F_RX][s]) + __ldg(&rec->pad[0]),
-                                           ((double)F[F_AX + 1][s] + F[F_RX + 1][s]) + __ldg(&rec->pad[1]),
-                                           ((double)F[F_AX + 2][s] + F[F_RX + 2][s]) + __ldg(&rec->pad[2]));
-            const double3 vd = make_double3((double)m.x - A.x, (double)m.y - A.y, (double)m.z - A.z);
-            bool in = true;
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-              double3 nd = make_double3((double)F[F_N0 + 3 * j][s] + __ldg(&rec->nlo[3 * j]),
-                                        (double)F[F_N0 + 3 * j + 1][s] + __ldg(&rec->nlo[3 * j + 1]),
-                                        (double)F[F_N0 + 3 * j + 2][s] + __ldg(&rec->nlo[3 * j + 2]));
-              in = in && dot3(nd, vd) >= 0.0;
-            }
-            if (in) {
-              const SceneView &V = kBatch ? a.views[__float_as_int(F[F_VI][s])] : a.v;
-              int s_slot = __float_as_int(__ldg(&rec->n0.w)), e_slot = __float_as_int(__ldg(&rec->n1.w));
-              float3 ns = make_float3(F[F_NS][s], F[F_NS + 1][s], F[F_NS + 2][s]);
-              float3 ne = make_float3(F[F_NE][s], F[F_NE + 1][s], F[F_NE + 2][s]);
-              double fs = s_slot >= 0 ? plane_side64(V, s_slot, ns, m) : 1.0;
-              double fe = e_slot >= 0 ? plane_side64(V, e_slot, ne, m) : 1.0;
-              in = fs > 0.0 && fe >= 0.0;
-            }
-            const double d2 = dot3(vd, vd);
-            if (in && d2 > 1e-18) {
-              const double gf = 1.0 / (4.0 * 3.141592653589793 * d2);
-              const double dist = has_alpha ? sqrt(d2) : 0.0;
-              const float *alpha = (kBatch ? a.views[__float_as_int(F[F_VI][s])] : a.v).alpha_log2;
-              double *e = energy + (size_t)mi * kMaxBands;
-#pragma unroll
-              for (int b = 0; b < kMaxBands; b++) {
-                if (b < nb) {
-                  double cval = (double)F[F_P + b][s] * gf;
-                  if (has_alpha) cval *= exp2((double)alpha[b] * dist);
-                  atomicAdd(e + b, cval);
-                }
-              }
-              atomicAdd(count + mi, 1);
-              n_contrib++;
-            }
-            continue;
-          }
           // m - apex with the apex as hi + lo: one extra rounding at most
           float3 v = make_float3((m.x - F[F_AX][s]) - F[F_RX][s], (m.y - F[F_AX + 1][s]) - F[F_RX + 1][s],
                                  (m.z - F[F_AX + 2][s]) - F[F_RX + 2][s]);
           n_cand++;
+          if (kF64) {
+            // FP64: a candidate that float32 finds outside by more than its
+            // rounding (four times its bound on a cone plane) is outside; the
+            // rest wait for float64
+            const float v1 = fabsf(v.x) + fabsf(v.y) + fabsf(v.z), side = 1e-3f + 4e-6f * v1;
+            near = true;
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+              const float3 nj = make_float3(F[F_N0 + 3 * j][s], F[F_N0 + 3 * j + 1][s], F[F_N0 + 3 * j + 2][s]);
+              near = near && dot3(nj, v) >= -2e-6f * v1 * (fabsf(nj.x) + fabsf(nj.y) + fabsf(nj.z));
+            }
+            const float3 ns = make_float3(F[F_NS][s], F[F_NS + 1][s], F[F_NS + 2][s]);
+            const float3 ne = make_float3(F[F_NE][s], F[F_NE + 1][s], F[F_NE + 2][s]);
+            near = near && dot3(ns, v) - F[F_NS + 3][s] >= -side && dot3(ne, v) - F[F_NE + 3][s] >= -side;
+            if (near) entry = make_int2(mi, __float_as_int(F[F_SI][s]));
+          } else {
           // cone planes: float32; within the rounding band of a plane the
           // test is redone with float pairs
           const float band_v = 2e-6f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z));
@@ -485,6 +515,20 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
             atomicAdd(&count[mi], 1);
             n_contrib++;
           }
+          }
+        }
+        if (kF64) {
+          const unsigned b = __ballot_sync(0xffffffffu, near);
+          if (near) wait[n_wait + __popc(b & ((1u << lane) - 1u))] = entry;
+          n_wait += __popc(b);
+          if (n_wait >= 32) {
+            __syncwarp();
+            n_contrib += contribute64<kBatch>(a, wait[lane]);
+            n_wait -= 32;
+            const int2 rest = wait[32 + lane];
+            __syncwarp();
+            wait[lane] = rest;
+          }
         }
       }
     }
@@ -493,6 +537,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
     base = (long long)__shfl_sync(0xffffffffu, taken, 0);
     lg = lg_next;
   }
+  if (kF64 && (int)lane < n_wait) n_contrib += contribute64<kBatch>(a, wait[lane]);
   for (int o = 16; o > 0; o >>= 1) {
     n_cand += __shfl_xor_sync(0xffffffffu, n_cand, o);
     n_contrib += __shfl_xor_sync(0xffffffffu, n_contrib, o);
