@@ -874,9 +874,7 @@ BT_API int bt_set_microphones(bt_ctx *c, int32_t scene_id, const float *pos, int
   TRY(ensure(c, s->energy, sizeof(double) * bt::kMaxBands * (size_t)n_m));
   TRY(ensure(c, s->count, sizeof(int) * (size_t)n_m));
   // the result accumulators start at zero (bt_trace_ranges may add to them)
-  CK(cudaMemsetAsync(s->energy.p, 0, sizeof(double) * bt::kMaxBands * (size_t)n_m, c->stream));
-  CK(cudaMemsetAsync(s->count.p, 0, sizeof(int) * (size_t)n_m, c->stream));
-  TRY(reset_counters(c));
+  CK(bt::launch_clear(st, (double *)s->energy.p, (int *)s->count.p, n_m, c->d_ctr, c->d_seg_count, c->n_sm));
   if (n_m > 0) CK(cudaMemcpyAsync(c->stage_a.p, pos, sizeof(float) * 3 * n_m, cudaMemcpyDefault, st));
   CK(bt::mic_box(st, (const float *)c->stage_a.p, n_m, c->d_box, &c->d_ctr->error));
   float box[6] = {0, 0, 0, 0, 0, 0};
