@@ -528,6 +528,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
             const int2 rest = wait[32 + lane];
             __syncwarp();
             wait[lane] = rest;
+            __syncwarp();
           }
         }
       }
@@ -537,6 +538,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
     base = (long long)__shfl_sync(0xffffffffu, taken, 0);
     lg = lg_next;
   }
+  __syncwarp();
   if (kF64 && (int)lane < n_wait) n_contrib += contribute64<kBatch>(a, wait[lane]);
   for (int o = 16; o > 0; o >>= 1) {
     n_cand += __shfl_xor_sync(0xffffffffu, n_cand, o);

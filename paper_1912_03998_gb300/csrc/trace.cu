@@ -655,7 +655,9 @@ __device__ __forceinline__ void search_phase(const DevScene &sc, bool lane_tris,
     run = __ballot_sync(0xffffffffu, more);
     if (kPairs) {
       __syncwarp();
-      const int n = *(volatile int *)wp.n;
+      // (one lane's reading for all: no lane may go on to the next step's
+      // additions before every lane has it, and all must decide alike)
+      const int n = __shfl_sync(0xffffffffu, *(volatile int *)wp.n, 0);
       // (the phase's end flushes, so that every lane without nodes is done)
       if (n >= kPairTest || (n > 0 && __popc(run) <= few))
         test_pairs<kP, kCount, kLeaves>(wp, n, tris, lane_tris, t_eps, dns, rs, dns64, hs, n_tris, tlim);
