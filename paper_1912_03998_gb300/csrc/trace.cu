@@ -1264,7 +1264,7 @@ constexpr int kRefillLanes = 28;
 //
 // Each warp alternates two phases.  In the search phase every lane with a ray
 // steps through the BVH one node at a time and the warp tests the triangles
-// they expose (by pairs: district unsplit 32.8 -> 29.0 ms together with the
+// they expose (by pairs: district unsplit 32.8 -> 28.6 ms together with the
 // near/far slab test and the wider-first nodes, FP64 on 24 of its sources
 // 8.4 -> 4.8 ms a call); the phase ends once kRefillLanes lanes have nothing to
 // search (their search finished, or they need a new lineage) or no lane is
