@@ -261,7 +261,8 @@ int bt_read_levels(bt_ctx *ctx, int32_t scene_id, double *level_db, double *inte
  *                  normalised ray to the hit triangle's plane), +inf on a miss
  *   tri_out        [n] int32 index of the hit triangle in the scene's input
  *                  order, -1 on a miss; equal distances go to the lowest index
- * Hits with distance <= t_eps_m are ignored. */
+ * Hits with distance <= t_eps_m are ignored.  A ray whose origin or direction
+ * is not finite, or whose direction is zero, hits nothing. */
 int bt_cast_rays(bt_ctx *ctx, int32_t scene_id, const float *origins, const float *dirs,
                  const float *start_normals, int64_t n, float t_eps_m, float *t_out,
                  int32_t *tri_out);

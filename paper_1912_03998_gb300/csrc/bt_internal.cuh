@@ -33,7 +33,7 @@ struct __align__(16) Node {
 
 // 4-wide node, 128 bytes (one cache line), what the traversal reads: the
 // boxes of up to four children, lane c of each float4 for child c, and their
-// codes (as in Node; kNoChild for an unused lane, whose box no ray meets).
+// codes (as in Node; kNoChild for an unused lane, whose box no finite ray meets).
 // Wide node i stands for binary node i: of the subtree below it the boxes that
 // are left when its children are opened, largest first, until there are four
 // (k_widen), so a traversal may start from any binary node.  Opening the
@@ -414,7 +414,9 @@ __device__ __forceinline__ bool slab(const Ray &r, float3 oi, float lox, float h
 }
 // The same with each axis' near and far plane told apart by the caller (by the
 // sign of the ray's direction): six fewer minima and maxima a box, the same
-// bounds.  An unused lane's inverted infinite box is missed by every ray.
+// bounds.  An unused lane's inverted infinite box is missed by every ray
+// without a NaN.  A NaN origin meets every box (PTX minima and maxima drop NaN),
+// so what would test an unused lane's code as a leaf checks for kNoChild.
 __device__ __forceinline__ bool slab_nf(float3 inv, float3 oi, float nx, float fx, float ny, float fy, float nz,
                                         float fz, float tmax, float &tnear) {
   const float tn = fmax3(fmaf(nx, inv.x, -oi.x), fmaf(ny, inv.y, -oi.y), fmaxf(fmaf(nz, inv.z, -oi.z), 0.0f));

@@ -467,11 +467,12 @@ __device__ __forceinline__ void test_pairs(const WarpPairs &wp, int n, const Tri
   const int lane = (int)lane_id();
   volatile int *const mail = wp.code;
   for (int base = 0; base < n; base += 32) {
-    const bool have = base + lane < n;
+    bool have = base + lane < n;
     int code = 0, owner = lane;
     if (have) {
       code = wp.code[base + lane];
       owner = wp.lane[base + lane];
+      have = code != ~kNoChild;  // (an unused lane, met by a NaN ray)
     }
     __syncwarp();
     RaySrc qs = rs;
@@ -606,6 +607,8 @@ __device__ __forceinline__ void search_phase(const DevScene &sc, bool lane_tris,
       const bool h2 = slab_nf(inv, oi, nx.z, fx.z, ny.z, fy.z, nz.z, fz.z, tmax, k2);
       const bool h3 = slab_nf(inv, oi, nx.w, fx.w, ny.w, fy.w, nz.w, fz.w, tmax, k3);
       int c0 = ch.x, c1 = ch.y, c2 = ch.z, c3 = ch.w;
+      // (to a NaN ray an unused lane looks like a leaf: test_pairs tells them
+      // apart, and without pairs no NaN ray is searched)
       const bool l0 = h0 && c0 < 0, l1 = h1 && c1 < 0, l2 = h2 && c2 < 0, l3 = h3 && c3 < 0;
       if (kPairs) {
         const int cnt = (int)l0 + (int)l1 + (int)l2 + (int)l3;
@@ -1787,7 +1790,9 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
       // is the ray's first, and a ray with none goes on to the next tile.
       const Ray r = make_ray(ld_hi3(sm, kRowO, t), ld_hi3(sm, kRowD, t), v.t_eps, ls.dns);
       tlim = tile_exit(tg, tile % tg.tx, tile / tg.tx, r) + kTileEps;
-      hs.start(__ldg(&ta.roots[tile]), v.sc.n_tris);
+      // (a ray that has become NaN hits nothing; search_phase by single lanes
+      // would take an unused lane of a node for a leaf of its)
+      hs.start(isnan(r.o.x + r.o.y + r.o.z) ? kNoChild : __ldg(&ta.roots[tile]), v.sc.n_tris);
       if constexpr (kDefer) rs.pend[0] = 0;
       more = true;
     }
@@ -1939,7 +1944,8 @@ __global__ void __launch_bounds__(128) k_cast(DevScene sc, const float *o, const
   int stack[kStackDepth];
   HitSearch hs;
   hs.start(sc.root, sc.n_tris);
-  bool more = mine;
+  // a ray with a NaN or infinite origin or direction hits nothing
+  bool more = mine && isfinite(O.x) && isfinite(O.y) && isfinite(O.z) && isfinite(Dd.x) && isfinite(Dd.y) && isfinite(Dd.z);
   search_phase<kPMixed, false, true, true>(sc, false, r, rs, dns, stack, err, hs, more, wp, none, none, kInf, 0);
   if (!mine) return;
   Best &best = hs.best;
