@@ -758,8 +758,11 @@ __device__ __forceinline__ void search_groups(const DevScene &sc, bool lane_tris
       const int total = __popc(ib);
       sp += total - take;
       // a well-formed BVH is visited at most once per node; the bound only
-      // guarantees termination should the structure ever be malformed
-      if (sp > kGroupDepth || __shfl_sync(kAll, hs.budget -= take, leader) < 0) {
+      // guarantees termination should the structure ever be malformed.  (The
+      // shuffle before the branch: sp differs between a warp's groups.)
+      hs.budget -= take;
+      const int budget = __shfl_sync(kAll, hs.budget, leader);
+      if (sp > kGroupDepth || budget < 0) {
         if (lane == leader) atomicExch(err, sp > kGroupDepth ? BT_E_QUEUE_FULL : BT_E_TIMEOUT);
         sp = 0;
       } else if (inner) {
