@@ -1693,10 +1693,13 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
           else if (r.d.x < 0.0f) tex = (tg.gx0 + ix * tg.wx - r.o.x) * r.inv.x;
           if (r.d.y > 0.0f) tey = (tg.gy0 + (iy + 1) * tg.wy - r.o.y) * r.inv.y;
           else if (r.d.y < 0.0f) tey = (tg.gy0 + iy * tg.wy - r.o.y) * r.inv.y;
-          leaves = tex == kInf && tey == kInf;
+          // (a ray that has become NaN leaves too: it has no next tile, and
+          // would be handed to its own without end)
+          const bool sx = tex <= tey, sy = tey <= tex;
+          leaves = (tex == kInf && tey == kInf) || !(sx || sy);
           if (!leaves) {
-            if (tex <= tey) ix += r.d.x > 0.0f ? 1 : -1;
-            if (tey <= tex) iy += r.d.y > 0.0f ? 1 : -1;
+            if (sx) ix += r.d.x > 0.0f ? 1 : -1;
+            if (sy) iy += r.d.y > 0.0f ? 1 : -1;
             leaves = ix < 0 || ix >= tg.tx || iy < 0 || iy >= tg.ty;
           }
           if (leaves || root_reachable(ta.bin, __ldg(&ta.roots[iy * tg.tx + ix]), r)) break;
