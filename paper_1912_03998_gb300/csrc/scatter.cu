@@ -669,157 +669,99 @@ cudaError_t launch_scatter(cudaStream_t st, const ScatterArgs &a, int n_sm) {
 // Tang, "Table-driven implementation of the logarithm function", 1990):
 // I = 2^e m with c ~ 1/m from the mantissa's seven leading bits, r = m c - 1
 // (|r| < 2^-8, one fused multiply-add), L = 10 log10(2) e + (120 - 10 log10 c)
-// + 10 log10(1 + r), the series' terms from r^4 on in float32.  That is 10
+// + 10 log10(1 + r), the series' terms from r^4 on in float32.  The two large
+// terms are split so that their leading parts add without rounding, and all
+// else is below 0.02: one rounding at the size of the result.  That is 10
 // float64 operations against some 35 of the library logarithm, and float64
 // issue is what bounds this kernel on GB300 (13.75 M microphones x 8 bands:
 // 6.7 ms, 0.4 ms of it memory).  Against 50-digit arithmetic over 1e-18..1e2
-// W/m^2 its error is 5.8e-15 dB (root mean square; the rounded 10 log10(I) + 120
-// has 6.1e-15).
-__device__ const double2 c_level_tab[128] = {  // c and 120 - 10 log10(c)
-    {0x1.fe01fe0000000p-1, 0x1.e01156832e30ep+6},
-    {0x1.fa11ca0000000p-1, 0x1.e033cffaf8abdp+6},
-    {0x1.f6310a0000000p-1, 0x1.e056058b502e6p+6},
-    {0x1.f25f640000000p-1, 0x1.e077f83b4e7c8p+6},
-    {0x1.ee9c800000000p-1, 0x1.e099a91277d83p+6},
-    {0x1.eae8080000000p-1, 0x1.e0bb19183bb8bp+6},
-    {0x1.e741aa0000000p-1, 0x1.e0dc494132c31p+6},
-    {0x1.e3a9180000000p-1, 0x1.e0fd3a6dee667p+6},
-    {0x1.e01e020000000p-1, 0x1.e11deda15a5eep+6},
-    {0x1.dca01e0000000p-1, 0x1.e13e63b6ed6b0p+6},
-    {0x1.d92f220000000p-1, 0x1.e15e9d992a97cp+6},
-    {0x1.d5cac80000000p-1, 0x1.e17e9c1be8e9fp+6},
-    {0x1.d272ca0000000p-1, 0x1.e19e60213ea9bp+6},
-    {0x1.cf26e60000000p-1, 0x1.e1bdea733b7a6p+6},
-    {0x1.cbe6da0000000p-1, 0x1.e1dd3be95c239p+6},
-    {0x1.c8b2660000000p-1, 0x1.e1fc555531015p+6},
-    {0x1.c5894e0000000p-1, 0x1.e21b376e32e15p+6},
-    {0x1.c26b540000000p-1, 0x1.e239e30bc317ep+6},
-    {0x1.bf583e0000000p-1, 0x1.e25858ea505a9p+6},
-    {0x1.bc4fd60000000p-1, 0x1.e27699aa17421p+6},
-    {0x1.b951e20000000p-1, 0x1.e294a61e7f87fp+6},
-    {0x1.b65e2e0000000p-1, 0x1.e2b27eea1ebebp+6},
-    {0x1.b374840000000p-1, 0x1.e2d024ce7c03ap+6},
-    {0x1.b094b40000000p-1, 0x1.e2ed985a97818p+6},
-    {0x1.adbe880000000p-1, 0x1.e30ada65273afp+6},
-    {0x1.aaf1d20000000p-1, 0x1.e327eb7ce30e5p+6},
-    {0x1.a82e660000000p-1, 0x1.e344cc24cb8e1p+6},
-    {0x1.a574100000000p-1, 0x1.e3617d3d16c40p+6},
-    {0x1.a2c2a80000000p-1, 0x1.e37dff3196126p+6},
-    {0x1.a01a020000000p-1, 0x1.e39a52a0b8cd3p+6},
-    {0x1.9d79f20000000p-1, 0x1.e3b67831f5576p+6},
-    {0x1.9ae24e0000000p-1, 0x1.e3d2708036507p+6},
-    {0x1.9852f00000000p-1, 0x1.e3ee3c0376b69p+6},
-    {0x1.95cbb00000000p-1, 0x1.e409db513957cp+6},
-    {0x1.934c680000000p-1, 0x1.e4254ef12bf6ap+6},
-    {0x1.90d4f20000000p-1, 0x1.e4409772bab3bp+6},
-    {0x1.8e65280000000p-1, 0x1.e45bb56d201acp+6},
-    {0x1.8bfce80000000p-1, 0x1.e476a9528895ap+6},
-    {0x1.899c100000000p-1, 0x1.e491739bf7b08p+6},
-    {0x1.87427c0000000p-1, 0x1.e4ac14e0124acp+6},
-    {0x1.84f00c0000000p-1, 0x1.e4c68d8f3fa60p+6},
-    {0x1.82a4a00000000p-1, 0x1.e4e0de205dd17p+6},
-    {0x1.8060180000000p-1, 0x1.e4fb0710cf0c1p+6},
-    {0x1.7e22560000000p-1, 0x1.e51508cd403d6p+6},
-    {0x1.7beb3a0000000p-1, 0x1.e52ee3dfda622p+6},
-    {0x1.79baa60000000p-1, 0x1.e54898c1e47fep+6},
-    {0x1.7790820000000p-1, 0x1.e56227abc4531p+6},
-    {0x1.756cac0000000p-1, 0x1.e57b91518caaep+6},
-    {0x1.734f0c0000000p-1, 0x1.e594d5f6e2d99p+6},
-    {0x1.7137860000000p-1, 0x1.e5adf61445e62p+6},
-    {0x1.6f26020000000p-1, 0x1.e5c6f1f78db05p+6},
-    {0x1.6d1a620000000p-1, 0x1.e5dfca3c68289p+6},
-    {0x1.6b14900000000p-1, 0x1.e5f87f22f2007p+6},
-    {0x1.6914740000000p-1, 0x1.e611110833521p+6},
-    {0x1.6719f40000000p-1, 0x1.e6298066d6d2cp+6},
-    {0x1.6524f80000000p-1, 0x1.e641cda611dfdp+6},
-    {0x1.63356c0000000p-1, 0x1.e659f8fff58f4p+6},
-    {0x1.614b360000000p-1, 0x1.e67202fdfca0bp+6},
-    {0x1.5f66440000000p-1, 0x1.e689ebc9ef6b4p+6},
-    {0x1.5d867c0000000p-1, 0x1.e6a1b3f6c8992p+6},
-    {0x1.5babcc0000000p-1, 0x1.e6b95bb6cac89p+6},
-    {0x1.59d6200000000p-1, 0x1.e6d0e3596907bp+6},
-    {0x1.5805600000000p-1, 0x1.e6e84b65d6d23p+6},
-    {0x1.56397c0000000p-1, 0x1.e6ff94007a94cp+6},
-    {0x1.54725e0000000p-1, 0x1.e716bd9f1efbep+6},
-    {0x1.52aff60000000p-1, 0x1.e72dc86d71e11p+6},
-    {0x1.50f22e0000000p-1, 0x1.e744b4e963bc9p+6},
-    {0x1.4f38f60000000p-1, 0x1.e75b8346054aep+6},
-    {0x1.4d843c0000000p-1, 0x1.e77233d4315a2p+6},
-    {0x1.4bd3ee0000000p-1, 0x1.e788c6e873014p+6},
-    {0x1.4a27fa0000000p-1, 0x1.e79f3cdb0bd18p+6},
-    {0x1.4880520000000p-1, 0x1.e7b595d1d3312p+6},
-    {0x1.46dce40000000p-1, 0x1.e7cbd22bb9247p+6},
-    {0x1.453d9e0000000p-1, 0x1.e7e1f24b75d2bp+6},
-    {0x1.43a2740000000p-1, 0x1.e7f7f6451c68bp+6},
-    {0x1.420b520000000p-1, 0x1.e80dde9d6b9a1p+6},
-    {0x1.40782e0000000p-1, 0x1.e823ab52c04e6p+6},
-    {0x1.3ee8f40000000p-1, 0x1.e8395cf09c3fbp+6},
-    {0x1.3d5d9a0000000p-1, 0x1.e84ef37ace303p+6},
-    {0x1.3bd60e0000000p-1, 0x1.e8646f6785de4p+6},
-    {0x1.3a52440000000p-1, 0x1.e879d0dbfb7e2p+6},
-    {0x1.38d22e0000000p-1, 0x1.e88f181c26631p+6},
-    {0x1.3755be0000000p-1, 0x1.e8a4456eddcbcp+6},
-    {0x1.35dce60000000p-1, 0x1.e8b9591ddd603p+6},
-    {0x1.34679a0000000p-1, 0x1.e8ce5358f2928p+6},
-    {0x1.32f5ce0000000p-1, 0x1.e8e334524cefap+6},
-    {0x1.3187760000000p-1, 0x1.e8f7fc3e824d7p+6},
-    {0x1.301c820000000p-1, 0x1.e90cab8f115a7p+6},
-    {0x1.2eb4ea0000000p-1, 0x1.e921424375283p+6},
-    {0x1.2d50a00000000p-1, 0x1.e935c0b513442p+6},
-    {0x1.2bef980000000p-1, 0x1.e94a2722aacedp+6},
-    {0x1.2a91ca0000000p-1, 0x1.e95e7591e0475p+6},
-    {0x1.2937260000000p-1, 0x1.e972ac817378cp+6},
-    {0x1.27dfa40000000p-1, 0x1.e986cbfb7c521p+6},
-    {0x1.268b380000000p-1, 0x1.e99ad447e626bp+6},
-    {0x1.2539d80000000p-1, 0x1.e9aec592cef58p+6},
-    {0x1.23eb7a0000000p-1, 0x1.e9c2a00a54f14p+6},
-    {0x1.22a0120000000p-1, 0x1.e9d663fd346bfp+6},
-    {0x1.2157980000000p-1, 0x1.e9ea117f407c2p+6},
-    {0x1.2012020000000p-1, 0x1.e9fda8c4ab22fp+6},
-    {0x1.1ecf440000000p-1, 0x1.ea112a22b60d6p+6},
-    {0x1.1d8f560000000p-1, 0x1.ea2495b2f2545p+6},
-    {0x1.1c52300000000p-1, 0x1.ea37eb9078bc9p+6},
-    {0x1.1b17c60000000p-1, 0x1.ea4b2c16c2d3cp+6},
-    {0x1.19e0120000000p-1, 0x1.ea5e574543c4ap+6},
-    {0x1.18ab080000000p-1, 0x1.ea716d7b85a33p+6},
-    {0x1.1778a20000000p-1, 0x1.ea846ebc410d9p+6},
-    {0x1.1648d60000000p-1, 0x1.ea975b4b252b3p+6},
-    {0x1.151b9a0000000p-1, 0x1.eaaa336e03f56p+6},
-    {0x1.13f0e80000000p-1, 0x1.eabcf72c5d86ap+6},
-    {0x1.12c8b80000000p-1, 0x1.eacfa6af22212p+6},
-    {0x1.11a3020000000p-1, 0x1.eae24220e1371p+6},
-    {0x1.107fbc0000000p-1, 0x1.eaf4c9ce6f95cp+6},
-    {0x1.0f5ee00000000p-1, 0x1.eb073dc543b4cp+6},
-    {0x1.0e40660000000p-1, 0x1.eb199e34d875ep+6},
-    {0x1.0d24460000000p-1, 0x1.eb2beb4e5102bp+6},
-    {0x1.0c0a780000000p-1, 0x1.eb3e25447af4cp+6},
-    {0x1.0af2f80000000p-1, 0x1.eb504c092d5c8p+6},
-    {0x1.09ddba0000000p-1, 0x1.eb626014a91cep+6},
-    {0x1.08cabc0000000p-1, 0x1.eb74613a028adp+6},
-    {0x1.07b9f20000000p-1, 0x1.eb864ff50091ap+6},
-    {0x1.06ab5a0000000p-1, 0x1.eb982c1ae60eep+6},
-    {0x1.059eea0000000p-1, 0x1.eba9f609087e4p+6},
-    {0x1.04949c0000000p-1, 0x1.ebbbaddabcb04p+6},
-    {0x1.038c6c0000000p-1, 0x1.ebcd538a41ef9p+6},
-    {0x1.0286500000000p-1, 0x1.ebdee779b40d8p+6},
-    {0x1.0182440000000p-1, 0x1.ebf069a5d8e26p+6},
-    {0x1.0080400000000p-1, 0x1.ec01da5179c5fp+6}};
+// W/m^2 its largest error is 1.42e-14 dB, half a unit in the last place, and its
+// root mean square 3.5e-15 (the rounded 10 log10(I) + 120: 1.47e-14 and 6.1e-15).
+struct LevelEntry {
+  double c, hi, lo;  // hi + lo = 120 - 10 log10(c), hi a multiple of 2^-17
+};
+__device__ const LevelEntry c_level_tab[128] = {
+    {0x1.fe01fep-1, 0x1.e01156p+6, 0x1.065c61b4a559ap-19}, {0x1.fa11cap-1, 0x1.e033dp+6, -0x1.41d50cee7acccp-24},
+    {0x1.f6310ap-1, 0x1.e05606p+6, -0x1.d2bf4682256fcp-20}, {0x1.f25f64p-1, 0x1.e077f8p+6, 0x1.da73e3c8d5202p-21},
+    {0x1.ee9c8p-1, 0x1.e099aap+6, -0x1.db104f983811fp-19}, {0x1.eae808p-1, 0x1.e0bb1ap+6, -0x1.cf888eac8a48bp-19},
+    {0x1.e741aap-1, 0x1.e0dc4ap+6, -0x1.7d9a79dd9c438p-19}, {0x1.e3a918p-1, 0x1.e0fd3ap+6, 0x1.b7b999b5145d1p-20},
+    {0x1.e01e02p-1, 0x1.e11deep+6, -0x1.7a96848d41e9ap-20}, {0x1.dca01ep-1, 0x1.e13e64p+6, -0x1.244a53ef3e708p-20},
+    {0x1.d92f22p-1, 0x1.e15e9ep+6, -0x1.9b55a0e639356p-20}, {0x1.d5cac8p-1, 0x1.e17e9cp+6, 0x1.be8e9f4b58e98p-22},
+    {0x1.d272cap-1, 0x1.e19e6p+6, 0x1.09f54d7654a34p-21}, {0x1.cf26e6p-1, 0x1.e1bdeap+6, 0x1.ccede9987c72dp-20},
+    {0x1.cbe6dap-1, 0x1.e1dd3cp+6, -0x1.6a3dc703daca1p-22}, {0x1.c8b266p-1, 0x1.e1fc56p+6, -0x1.559dfd69877f7p-19},
+    {0x1.c5894ep-1, 0x1.e21b38p+6, -0x1.239a3d6aea982p-19}, {0x1.c26b54p-1, 0x1.e239e4p+6, -0x1.e879d03304b59p-19},
+    {0x1.bf583ep-1, 0x1.e25858p+6, 0x1.d4a0b519628b5p-19}, {0x1.bc4fd6p-1, 0x1.e2769ap+6, -0x1.57a2f7cfc0eb1p-20},
+    {0x1.b951e2p-1, 0x1.e294a6p+6, 0x1.e7f87e8ed1c89p-22}, {0x1.b65e2ep-1, 0x1.e2b27ep+6, 0x1.d43d7d5ba5d91p-19},
+    {0x1.b37484p-1, 0x1.e2d024p+6, 0x1.9cf8074397a42p-19}, {0x1.b094b4p-1, 0x1.e2ed98p+6, 0x1.6a5e061fb7f08p-20},
+    {0x1.adbe88p-1, 0x1.e30adap+6, 0x1.949ceba3fdf9cp-20}, {0x1.aaf1d2p-1, 0x1.e327ecp+6, -0x1.0639e36e5fe89p-19},
+    {0x1.a82e66p-1, 0x1.e344ccp+6, 0x1.265c70ae2b138p-21}, {0x1.a5741p-1, 0x1.e3617ep+6, -0x1.85d27808810d4p-19},
+    {0x1.a2c2a8p-1, 0x1.e37ep+6, -0x1.9cd3db43aeeddp-19}, {0x1.a01a02p-1, 0x1.e39a52p+6, 0x1.41719a6de3314p-19},
+    {0x1.9d79f2p-1, 0x1.e3b678p+6, 0x1.8faabaf5162e1p-21}, {0x1.9ae24ep-1, 0x1.e3d27p+6, 0x1.006ca0ef1c38ep-19},
+    {0x1.9852fp-1, 0x1.e3ee3cp+6, 0x1.bb5b477aab93dp-25}, {0x1.95cbbp-1, 0x1.e409dcp+6, -0x1.5d8d508d107a8p-19},
+    {0x1.934c68p-1, 0x1.e4254ep+6, 0x1.e257ed31d20b4p-19}, {0x1.90d4f2p-1, 0x1.e44098p+6, -0x1.1a8a98a09a905p-19},
+    {0x1.8e6528p-1, 0x1.e45bb6p+6, -0x1.25bfca82973dep-19}, {0x1.8bfce8p-1, 0x1.e476aap+6, -0x1.5aeed4b8f38e3p-19},
+    {0x1.899c1p-1, 0x1.e49174p+6, -0x1.90213df5004a7p-20}, {0x1.87427cp-1, 0x1.e4ac14p+6, 0x1.c0249582c54dcp-19},
+    {0x1.84f00cp-1, 0x1.e4c68ep+6, -0x1.c301680e76de8p-20}, {0x1.82a4ap-1, 0x1.e4e0dep+6, 0x1.02ee8b5dfa635p-21},
+    {0x1.806018p-1, 0x1.e4fb08p+6, -0x1.de61e7e665f21p-19}, {0x1.7e2256p-1, 0x1.e51508p+6, 0x1.9a807acfc9931p-19},
+    {0x1.7beb3ap-1, 0x1.e52ee4p+6, -0x1.012cef0926b4p-21}, {0x1.79baa6p-1, 0x1.e54898p+6, 0x1.83c8ffcf9a001p-19},
+    {0x1.779082p-1, 0x1.e56228p+6, -0x1.50eeb3aa18876p-20}, {0x1.756cacp-1, 0x1.e57b92p+6, -0x1.5ce6aa3b9e3a9p-19},
+    {0x1.734f0cp-1, 0x1.e594d6p+6, -0x1.23a4ce871f33dp-23}, {0x1.713786p-1, 0x1.e5adf6p+6, 0x1.445e618da2e6p-22},
+    {0x1.6f2602p-1, 0x1.e5c6f2p+6, -0x1.0e49f57ce00acp-23}, {0x1.6d1a62p-1, 0x1.e5dfcap+6, 0x1.e34144b22c427p-21},
+    {0x1.6b149p-1, 0x1.e5f88p+6, -0x1.ba1bff2ec8fb9p-19}, {0x1.691474p-1, 0x1.e61112p+6, -0x1.ef995be98c7c5p-19},
+    {0x1.6719f4p-1, 0x1.e6298p+6, 0x1.9b5b4b005a7b6p-20}, {0x1.6524f8p-1, 0x1.e641cep+6, -0x1.67b880a5bdab4p-20},
+    {0x1.63356cp-1, 0x1.e659f8p+6, 0x1.ffeb1e8e9745bp-19}, {0x1.614b36p-1, 0x1.e67202p+6, 0x1.fbf9415459c13p-19},
+    {0x1.5f6644p-1, 0x1.e689ecp+6, -0x1.b084a62361978p-21}, {0x1.5d867cp-1, 0x1.e6a1b4p+6, -0x1.26ecdcf736fcep-23},
+    {0x1.5babccp-1, 0x1.e6b95cp+6, -0x1.24d4ddb955355p-20}, {0x1.59d62p-1, 0x1.e6d0e4p+6, -0x1.4d2df0977e1e3p-19},
+    {0x1.58056p-1, 0x1.e6e84cp+6, -0x1.34525bac141b2p-19}, {0x1.56397cp-1, 0x1.e6ff94p+6, 0x1.ea5305a613146p-28},
+    {0x1.54725ep-1, 0x1.e716bep+6, -0x1.8384107b4e8cbp-20}, {0x1.52aff6p-1, 0x1.e72dc8p+6, 0x1.b5c78450e3c43p-20},
+    {0x1.50f22ep-1, 0x1.e744b4p+6, 0x1.d2c77918cff35p-19}, {0x1.4f38f6p-1, 0x1.e75b84p+6, -0x1.73f56a3c7adbfp-19},
+    {0x1.4d843cp-1, 0x1.e77234p+6, -0x1.5e752f2c8ec57p-21}, {0x1.4bd3eep-1, 0x1.e788c6p+6, 0x1.d0e6028559568p-19},
+    {0x1.4a27fap-1, 0x1.e79f3cp+6, 0x1.b617a2f8c6157p-19}, {0x1.488052p-1, 0x1.e7b596p+6, -0x1.7166770a338fdp-21},
+    {0x1.46dce4p-1, 0x1.e7cbd2p+6, 0x1.5dc92392d2ce6p-21}, {0x1.453d9ep-1, 0x1.e7e1f2p+6, 0x1.2dd74abd67f6bp-20},
+    {0x1.43a274p-1, 0x1.e7f7f6p+6, 0x1.1471a2dedbb3p-20}, {0x1.420b52p-1, 0x1.e80ddep+6, 0x1.3ad734236971p-19},
+    {0x1.40782ep-1, 0x1.e823acp+6, -0x1.5a7f63374ed0ep-19}, {0x1.3ee8f4p-1, 0x1.e8395cp+6, 0x1.e1387f5c1991bp-19},
+    {0x1.3d5d9ap-1, 0x1.e84ef4p+6, -0x1.0a639f9846eb1p-19}, {0x1.3bd60ep-1, 0x1.e8647p+6, -0x1.30f443735abep-19},
+    {0x1.3a5244p-1, 0x1.e879dp+6, 0x1.b7f6fc4e53bbfp-19}, {0x1.38d22ep-1, 0x1.e88f18p+6, 0x1.c266311f596ap-22},
+    {0x1.3755bep-1, 0x1.e8a446p+6, -0x1.2244687a7a8f2p-19}, {0x1.35dce6p-1, 0x1.e8b95ap+6, -0x1.c4453fa984053p-19},
+    {0x1.34679ap-1, 0x1.e8ce54p+6, -0x1.4e1adaf23c834p-19}, {0x1.32f5cep-1, 0x1.e8e334p+6, 0x1.4933be6474213p-20},
+    {0x1.318776p-1, 0x1.e8f7fcp+6, 0x1.f4126b97fb48dp-21}, {0x1.301c82p-1, 0x1.e90cacp+6, -0x1.c3ba9642d0397p-20},
+    {0x1.2eb4eap-1, 0x1.e92142p+6, 0x1.0dd4a0c4597d2p-20}, {0x1.2d50ap-1, 0x1.e935cp+6, 0x1.6a268837f7ae2p-19},
+    {0x1.2bef98p-1, 0x1.e94a28p+6, -0x1.baaa6251f6cf9p-19}, {0x1.2a91cap-1, 0x1.e95e76p+6, -0x1.b87ee2d2959abp-20},
+    {0x1.293726p-1, 0x1.e972acp+6, 0x1.02e6f18a7a988p-19}, {0x1.27dfa4p-1, 0x1.e986ccp+6, -0x1.20eb7a5b1099ap-24},
+    {0x1.268b38p-1, 0x1.e99ad4p+6, 0x1.1f989ab0f5da4p-20}, {0x1.2539d8p-1, 0x1.e9aec6p+6, -0x1.b4c42a13b79f2p-20},
+    {0x1.23eb7ap-1, 0x1.e9c2ap+6, 0x1.4a9e27d91f3bap-23}, {0x1.22a012p-1, 0x1.e9d664p+6, -0x1.65ca05b7aa4dep-25},
+    {0x1.215798p-1, 0x1.e9ea12p+6, -0x1.017f07b3e44dp-19}, {0x1.201202p-1, 0x1.e9fda8p+6, 0x1.895645e783d7dp-19},
+    {0x1.1ecf44p-1, 0x1.ea112ap+6, 0x1.15b06b18f886bp-21}, {0x1.1d8f56p-1, 0x1.ea2496p+6, -0x1.3436aec5e4785p-20},
+    {0x1.1c523p-1, 0x1.ea37ecp+6, -0x1.be1d0db15b264p-20}, {0x1.1b17c6p-1, 0x1.ea4b2cp+6, 0x1.6c2d3b989528ep-22},
+    {0x1.19e012p-1, 0x1.ea5e58p+6, -0x1.757876b3d22aap-19}, {0x1.18ab08p-1, 0x1.ea716ep+6, -0x1.08f4b9a8d70c7p-19},
+    {0x1.1778a2p-1, 0x1.ea846ep+6, 0x1.78821b1d97036p-19}, {0x1.1648d6p-1, 0x1.ea975cp+6, -0x1.69b5a9a819ffep-19},
+    {0x1.151b9ap-1, 0x1.eaaa34p+6, -0x1.23f8154b11c7ep-19}, {0x1.13f0e8p-1, 0x1.eabcf8p+6, -0x1.a744f2cb316acp-19},
+    {0x1.12c8b8p-1, 0x1.eacfa6p+6, 0x1.5e44424cab5bdp-19}, {0x1.11a302p-1, 0x1.eae242p+6, 0x1.0709b84b5bafep-21},
+    {0x1.107fbcp-1, 0x1.eaf4cap+6, -0x1.8c8351c1e5262p-21}, {0x1.0f5eep-1, 0x1.eb073ep+6, -0x1.d5e259c8089ap-21},
+    {0x1.0e4066p-1, 0x1.eb199ep+6, 0x1.a6c3af2faa0c6p-21}, {0x1.0d2446p-1, 0x1.eb2becp+6, -0x1.635dfaa2dda05p-19},
+    {0x1.0c0a78p-1, 0x1.eb3e26p+6, -0x1.770a16843b19ep-19}, {0x1.0af2f8p-1, 0x1.eb504cp+6, 0x1.25ab9096cf361p-23},
+    {0x1.09ddbap-1, 0x1.eb626p+6, 0x1.4a91cdd27e1d3p-22}, {0x1.08cabcp-1, 0x1.eb7462p+6, -0x1.8bfaea606335cp-19},
+    {0x1.07b9f2p-1, 0x1.eb865p+6, -0x1.5fedcb1b43bf4p-23}, {0x1.06ab5ap-1, 0x1.eb982cp+6, 0x1.ae60edb965f84p-22},
+    {0x1.059eeap-1, 0x1.eba9f6p+6, 0x1.210fc73336283p-23}, {0x1.04949cp-1, 0x1.ebbbaep+6, -0x1.2a1a7e28925c3p-21},
+    {0x1.038c6cp-1, 0x1.ebcd54p+6, -0x1.d6f841d63da3ep-20}, {0x1.02865p-1, 0x1.ebdee8p+6, -0x1.0c97e507f5645p-19},
+    {0x1.018244p-1, 0x1.ebf06ap+6, -0x1.689c7675517b5p-20}, {0x1.00804p-1, 0x1.ec01dap+6, 0x1.45e717b058f0bp-20}};
 
 __device__ __forceinline__ double level_of(double I) {
   if (!(I > 0.0)) return -__builtin_huge_val();
   const unsigned long long u = (unsigned long long)__double_as_longlong(I);
   const int ex = (int)(u >> 52);
   if (ex == 0 || ex == 0x7ff) return 10.0 * log10(I) + 120.0;  // denormal or infinite
-  const double2 ct = __ldg(&c_level_tab[(int)(u >> 45) & 127]);
+  const LevelEntry *const ct = &c_level_tab[(int)(u >> 45) & 127];
   const double m = __longlong_as_double((long long)((u & 0xfffffffffffffull) | 0x3ff0000000000000ull));
-  const double r = fma(m, ct.x, -1.0);
+  const double r = fma(m, __ldg(&ct->c), -1.0);
   // 10 / ln 10, and 10 log10(2) in two parts, the first of 24 bits
   const double k = 0x1.15f2ced384f29p+2, hi = 0x1.815182p+1, lo = 0x1.31d61fabf59b6p-25;
   const float f = (float)r, kf = (float)k;
   const float t = f * fmaf(f, fmaf(f, -kf / 6.0f, kf / 5.0f), -kf / 4.0f);
   const double e = (double)(ex - 1023);
   const double p = fma(r, fma(r, k / 3.0 + (double)t, -k / 2.0), k);
-  return fma(e, hi, ct.y) + fma(e, lo, r * p);
+  // e hi + ct->hi is exact: multiples of 2^-22 below 2^12
+  return fma(e, hi, __ldg(&ct->hi)) + fma(r, p, fma(e, lo, __ldg(&ct->lo)));
 }
 
 // The outputs that are wanted, in the caller's microphone order.

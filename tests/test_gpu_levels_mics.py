@@ -61,3 +61,28 @@ def test_every_microphone_binned_once(n, kind):
     ref = w.power[0].astype(np.float64)[None] / (4.0 * np.pi * d2[:, None])
     # float32 distance and quotient: a few 2^-24 relative
     np.testing.assert_allclose(g["I"], ref, rtol=1e-6)
+
+
+def test_levels_are_rounded_once():
+    """Against 50-digit arithmetic: half a unit in the last place of the level,
+    and 1e-16 dB for all that the readout adds below it (its largest small part
+    is 0.02 dB, rounded a few times, and a float32 tail of 6e-17 dB)."""
+    from decimal import Decimal, localcontext
+    rng = np.random.default_rng(3)
+    n, nb = 500, 8
+    I = 10.0 ** rng.uniform(-18.0, 2.0, (n, nb))
+    I[:100] = 10.0 ** rng.uniform(-300.0, 300.0, (100, nb))
+    I[100:150] = 1e-12 * (1.0 + rng.uniform(-1e-3, 1e-3, (50, nb)))
+    w = synth.ground_only(level=1)
+    with btrace.Tracer(0) as t:
+        sid = btrace.bt_load_scene(t.ctx, w.scene.verts, w.scene.tris, w.scene.mat, synth.refl_table(n_bands=nb))
+        btrace.bt_set_microphones(t.ctx, sid, rng.uniform(-50.0, 50.0, (n, 3)).astype(np.float32))
+        btrace.bt_set_result(t.ctx, sid, I, np.zeros(n, np.int32))
+        L = np.empty((n, nb))
+        btrace.bt_read_levels(t.ctx, sid, L)
+    with localcontext() as ctx:
+        ctx.prec = 50
+        ref = [10 * Decimal(float(x)).log10() + 120 for x in I.ravel()]
+        err = np.array([abs(float(Decimal(float(y)) - r)) for y, r in zip(L.ravel(), ref)])
+    tol = 0.5 * np.spacing(np.abs(np.array([float(r) for r in ref]))) + 1e-16
+    assert (err <= tol).all(), (err / tol).max()
