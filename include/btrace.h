@@ -64,7 +64,9 @@ extern "C" {
  * BT_PREC_FP64: the image-source chain in float64; every triangle test in
  *   float64 (Moller-Trumbore on the float64 ray; the BVH boxes stay float32,
  *   grown to be conservative); every microphone test and contribution in
- *   float64 (the apex exact, cone normals to about 48 bits); band powers
+ *   float64 (the apex exact, cone normals to about 48 bits), but for
+ *   microphones that float32 finds outside by more than its own rounding (a
+ *   derived bound, free of the scene's extent); band powers
  *   W_b prod(r_b) in float32; float64 accumulation.  Slower: GB300 issues
  *   float64 at a small fraction of the float32 rate.
  * BT_PREC_MIXED64: float32 traversal and hit tests as in MIXED (ambiguous

@@ -13,8 +13,10 @@
 //
 // Precision.  Microphone tests are float32 relative to the apex and are
 // re-tested with float pairs when a microphone lies within the rounding band
-// of a cone or start/end plane (BT_PREC_MIXED and FP32), or run in float64
-// throughout (BT_PREC_FP64); intensity accumulates in float64.
+// of a cone or start/end plane (BT_PREC_MIXED and FP32).  In BT_PREC_FP64
+// float32 only sorts out what it finds outside by more than its rounding;
+// every other test and every contribution is float64.  Intensity accumulates
+// in float64.
 #include "bt_internal.cuh"
 
 namespace bt {
@@ -451,8 +453,15 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
           n_cand++;
           if (kF64) {
             // FP64: a candidate that float32 finds outside by more than its
-            // rounding (four times its bound on a cone plane) is outside; the
-            // rest wait for float64
+            // rounding is outside; the rest wait for float64.  With v the
+            // microphone from the apex, u = 2^-24 and |.| the sum of magnitudes:
+            // v and the normals n are rounded to u, a dot product of three
+            // terms to 3 u |n||v|, so a cone plane's value errs by at most
+            // 5 u |n||v| = 3e-7 |n||v| against 2e-6.  Start and end planes: the
+            // same with |n| < 1.8, and the offset, formed in float64 with the
+            // float64 normal, rounded to u of itself (within the slack, of at
+            // most 1.8 |v|): 7e-7 |v| against 4e-6 |v| + 1 mm, whatever the
+            // size of the triangle and its distance.
             const float v1 = fabsf(v.x) + fabsf(v.y) + fabsf(v.z), side = 1e-3f + 4e-6f * v1;
             near = true;
 #pragma unroll

@@ -1009,11 +1009,16 @@ __device__ __forceinline__ bool finish_segment(const TraceArgs &a, const SceneVi
     plf = __ldg(&v.sc.planes[slot]);
     // end plane on the incident side, offset relative to the apex
     float3 pn = f3(plf);
-    float3 en = dot3(pn, r.d) < 0.0f ? pn : pn * -1.0f;
+    const bool facing = dot3(pn, r.d) < 0.0f;
+    float3 en = facing ? pn : pn * -1.0f;
     float ew;
     if (kChain64) {
-      double3 end = make_double3(en.x, en.y, en.z);
-      ew = (float)dot3(end, make_double3(v0.x, v0.y, v0.z) - ld_d3(sm, kRowA, t));
+      // (with the float64 normal: the float32 one errs by its rounding times
+      // the distance to v0, which a triangle of many km makes centimetres, and
+      // FP64's scatter sorts microphones out by this offset)
+      const Plane64 pl = ldg_d4(&v.sc.planes64[slot]);
+      const double w = dot3(make_double3(pl.x, pl.y, pl.z), make_double3(v0.x, v0.y, v0.z) - ld_d3(sm, kRowA, t));
+      ew = (float)(facing ? w : -w);
     } else if (kPairs) {
       ew = df3_dot2(mkdf3(en), df3_sub(mkdf3(f3(v0)), ld_df3(sm, kRowA, t))).hi;
     } else {

@@ -176,3 +176,44 @@ def test_precision_matrix_district(tracer, oracle_mod):
     print("PRECISION_MATRIX " + json.dumps(rows))
     for name in ("mixed", "mixed64", "fp64"):
         assert rows[name]["frac_within_0p1"] >= 0.999 and rows[name]["max_db"] <= 1.0, (name, rows[name])
+
+
+@pytest.mark.parametrize("name", ["fp64", "mixed64"])
+def test_microphones_by_a_triangle_of_many_km(tracer, oracle_mod, name):
+    """Microphones up to 5 mm in front of a triangle whose first vertex is 1,000 km
+    away, so that the float32 rounding of its normal displaces its plane at the
+    microphones by more than a centimetre.  The seeds give planes displaced to
+    the microphones' side, where they would seem to lie behind the wall."""
+    found = 0
+    for seed in range(60):
+        rng = np.random.default_rng(seed)
+        az, tilt = rng.uniform(0.0, 2.0 * np.pi), rng.uniform(0.2, 0.6)
+        n = np.array([np.cos(az) * np.cos(tilt), np.sin(az) * np.cos(tilt), np.sin(tilt)])
+        u = np.cross(n, [0.0, 0.0, 1.0])
+        u /= np.linalg.norm(u)
+        v = np.cross(n, u)
+        verts = np.array([20 * n + 1e6 * u + 200 * v, 20 * n - 300 * u - 300 * v, 20 * n - 300 * u + 300 * v], np.float32)
+        a, b, c = verts.astype(np.float64)
+        nn = np.cross(b - a, c - a)
+        nn /= np.linalg.norm(nn)
+        e = (nn.astype(np.float32).astype(np.float64) - nn) @ (20 * n - a)
+        if abs(e) < 0.015:
+            continue
+        found += 1
+        front = -np.sign(e) * nn
+        foot = 20 * n - ((20 * n - a) @ nn) * nn
+        lat = rng.uniform(-15.0, 15.0, (400, 2))
+        mics = (foot + lat[:, :1] * u + lat[:, 1:] * v)
+        mics -= ((mics - a) @ nn)[:, None] * nn
+        mics = (mics + rng.uniform(0.0, 5e-3, (400, 1)) * front).astype(np.float32)
+        depth = (mics.astype(np.float64) - a) @ front
+        mics = mics[depth > 1e-4]  # (clear of both sides' rounding)
+        w = synth.ground_only(level=3)
+        w.scene.verts, w.scene.tris, w.scene.mat = verts, np.array([[0, 1, 2]], np.int32), np.zeros(1, np.uint8)
+        w.src, w.mics, w.max_order = (foot + 30.0 * front)[None].astype(np.float32), mics, 0
+        g = gpu_run(tracer, w, precision=prec(name))
+        r = oracle_mod.trace_workload(w)
+        assert (r["cnt"] == 1).all()
+        assert (g["cnt"] == r["cnt"]).all(), (seed, int((g["cnt"] != r["cnt"]).sum()))
+        np.testing.assert_allclose(g["I"], r["I"], rtol=2e-6)
+    assert found >= 3
