@@ -1861,6 +1861,10 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
 // split 4 x 4: 5,120 385/333/336/352, 40,960 968/634/767/966.  Not for the
 // float64 chain, which leaves too much to one lane of a group (FP64 at 10,240
 // lineages 344/245/332/541 and 225/249/374/623).
+// A warp of groups holds 32 >> log2 lineages, so it reserves that share of
+// beams_per_warp: with all of it a warp went through its reservation two at a
+// time while others had none (8 x 8-block city, 5,120 lineages, 256 a warp: 4.79
+// ms, by shares 0.35, single lanes 0.86).
 template <int kP>
 static int group_log2(int64_t n, int n_sm) {
   const int64_t lanes = (int64_t)n_sm * 7 * kTraceThreads;
@@ -1899,7 +1903,10 @@ static cudaError_t launch_tiled_p(cudaStream_t st, const TraceArgs &a0, const Ti
   // (FP32's chain rounds by each kernel's own contractions, so it keeps to the
   // kernel that larger launches run)
   if constexpr (kP == kPMixed)
-    if (a.group_log2 > 0) return launch_tiled_t<kP, false, false, true>(st, a, ta, n_sm);
+    if (a.group_log2 > 0) {
+      a.beams_per_warp >>= a.group_log2;
+      return launch_tiled_t<kP, false, false, true>(st, a, ta, n_sm);
+    }
   return launch_tiled_t<kP, false, false, false>(st, a, ta, n_sm);
 }
 
@@ -2010,7 +2017,10 @@ static cudaError_t launch_trace_p(cudaStream_t st, const TraceArgs &a0, int n_sm
                         : launch_trace_t<kP, false, kBatch, true, false>(st, a, n_sm);
   if (a.count_work) return launch_trace_t<kP, true, kBatch, false, false>(st, a, n_sm);
   if constexpr (!Prec<kP>::chain64)
-    if (a.group_log2 > 0) return launch_trace_t<kP, false, kBatch, false, true>(st, a, n_sm);
+    if (a.group_log2 > 0) {
+      a.beams_per_warp >>= a.group_log2;  // as many for each lineage that a warp holds
+      return launch_trace_t<kP, false, kBatch, false, true>(st, a, n_sm);
+    }
   return launch_trace_t<kP, false, kBatch, false, false>(st, a, n_sm);
 }
 
