@@ -1521,9 +1521,12 @@ __device__ __forceinline__ int take_handoffs(const TiledArgs &ta, int home, int 
 // lineages in flight.  A lineage in flight holds one of qcap credits; a warp
 // draws credits from the global count in chunks, keeps those of lineages
 // that end on it for its next fresh lineages, and gives back any above one
-// per lane.  Warp-collective, warp-uniform result: the first lineage offset
+// for each of the `slots` lineages it can hold (drawn for 32 by a warp of lane
+// groups, they starved the other warps of a launch with shallow queues: 8 x 8-
+// block city split 4 x 4, 40,960 lineages, depth 4,096: 2.51 ms, now 0.72, single
+// lanes 1.86).  Warp-collective, warp-uniform result: the first lineage offset
 // and the count; *exhausted is set once the batch is used up.
-__device__ __forceinline__ int take_fresh(const TraceArgs &a, const TiledArgs &ta, int want, int &credits,
+__device__ __forceinline__ int take_fresh(const TraceArgs &a, const TiledArgs &ta, int want, int slots, int &credits,
                                           int64_t &base, bool &exhausted, WarpLineages &wl) {
   int *used = ta.ctl + 3 * ta.n_tiles;
   int got = 0;
@@ -1536,7 +1539,7 @@ __device__ __forceinline__ int take_fresh(const TraceArgs &a, const TiledArgs &t
     // reservations never exceed the cap on lineages in flight
     const int bpw = a.beams_per_warp;
     const bool refill = bpw > 0 && wl.next == wl.end && !wl.last;
-    const int target = bpw > 32 ? bpw : 32;
+    const int target = bpw > slots ? bpw : slots;
     if (c < want || (refill && c < target)) {
       int req = target - c;
       int old = atomicAdd(used, req);
@@ -1639,6 +1642,7 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
   const int t = (int)threadIdx.x >> lg;
   const unsigned lane = lane_id();
   const bool lead = (lane & ((1u << lg) - 1u)) == 0u;  // (only a group's leader takes lineages)
+  const int slots = 32 >> lg;                          // lineages the warp can hold
   const unsigned below = (1u << lane) - 1u;
   const SceneView &v = a.v;
   const TileGrid &tg = ta.tg;  // read from parameter space, not held in registers
@@ -1723,7 +1727,7 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
     unsigned em = __ballot_sync(0xffffffffu, ended);
     if (em) {
       credits += __popc(em);
-      int give = credits > 32 ? credits - 32 : 0;
+      int give = credits > slots ? credits - slots : 0;
       credits -= give;
       if ((int)lane == __ffs(em) - 1) {
         if (give) atomicSub(used, give);
@@ -1781,7 +1785,7 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
       nm = __ballot_sync(0xffffffffu, lead && !active);
       if (nm && !exhausted) {
         int64_t fb;
-        int got_f = take_fresh(a, ta, __popc(nm), credits, fb, exhausted, wlin[threadIdx.x >> 5]);
+        int got_f = take_fresh(a, ta, __popc(nm), slots, credits, fb, exhausted, wlin[threadIdx.x >> 5]);
         int rank = __popc(nm & below);
         if (lead && !active && rank < got_f) {
           int64_t mine = a.lineage_begin + fb + rank;
@@ -1882,10 +1886,12 @@ static cudaError_t launch_tiled_t(cudaStream_t st, const TraceArgs &a, const Til
   if (per_sm < 1) per_sm = 1;
   int64_t blocks = (int64_t)n_sm * per_sm;
   if (kGroup) {
-    // no more blocks than lineages need: warps without work poll the queues,
-    // which slows a small launch down (5,120 lineages split 4 x 4: 262 -> 190 us)
+    // no more blocks than lineages need, all or (with shallow queues) those in
+    // flight: warps without work poll the queues, which slows a small launch
+    // down (5,120 lineages split 4 x 4: 262 -> 190 us)
     const int cols = kTraceThreads >> a.group_log2;
-    const int64_t need = (a.lineage_end - a.lineage_begin + cols - 1) / cols;
+    const int64_t all = a.lineage_end - a.lineage_begin, most = all < (int64_t)ta.qcap ? all : (int64_t)ta.qcap;
+    const int64_t need = (most + cols - 1) / cols;
     if (blocks > need) blocks = need;
   }
   k_trace_tiled<kP, kCount, kLeaves, kGroup><<<(int)blocks, kTraceThreads, 0, st>>>(a, ta);

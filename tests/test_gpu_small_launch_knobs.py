@@ -35,3 +35,8 @@ def check(city, sources, **kw):
 @pytest.mark.parametrize("sources,beams_per_warp", [(1, 32), (1, 256), (8, 64), (8, 1024)])
 def test_reserved_lineages(city, tiles, sources, beams_per_warp):
     check(city, sources, tiles_x=tiles, tiles_y=tiles, beams_per_warp=beams_per_warp)
+
+
+@pytest.mark.parametrize("sources,queue_depth", [(1, 32), (1, 1024), (2, 256), (8, 32), (8, 256), (8, 4096)])
+def test_shallow_queues(city, sources, queue_depth):
+    check(city, sources, tiles_x=4, tiles_y=4, queue_depth=queue_depth)
