@@ -1869,11 +1869,24 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
 // beams_per_warp: with all of it a warp went through its reservation two at a
 // time while others had none (8 x 8-block city, 5,120 lineages, 256 a warp: 4.79
 // ms, by shares 0.35, single lanes 0.86).
+// With fewer blocks per SM than fit (the blocks_per_sm knob) the lines move down:
+// unsplit with up to five, which do what seven do, split with all.  8 x 8-block
+// city, 1 / 8 / 16 lanes:
+//   1 block:  5,120 133/86/118, 10,240 135/143/217, 40,960 196/459/708
+//   2 blocks: 10,240 137/96/133, 20,480 143/155/231, 40,960 157/276/411
+//   split, 1 block:  5,120 167/147/192, 10,240 174/294/446, 40,960 262/849/1,288
+//   split, 2 blocks: 10,240 210/229/317, 20,480 217/360/520
 template <int kP>
-static int group_log2(int64_t n, int n_sm) {
-  const int64_t lanes = (int64_t)n_sm * 7 * kTraceThreads;
+static int group_log2(int64_t n, int n_sm, int blocks_per_sm, bool split) {
   if (Prec<kP>::chain64) return 0;
-  return n <= lanes / 16 ? 4 : (n <= lanes * 3 / 8 ? 3 : 0);
+  const int blocks = blocks_per_sm > 0 && blocks_per_sm < 7 ? blocks_per_sm : 7;
+  const int64_t sm_lanes = (int64_t)n_sm * kTraceThreads;
+  if (split) {
+    const int64_t lanes = sm_lanes * blocks;
+    return n <= lanes / 16 ? 4 : (n <= lanes * 3 / 8 ? 3 : 0);
+  }
+  const int64_t lanes = sm_lanes * (blocks < 5 ? blocks : 5);
+  return n <= lanes * 3 / 32 ? 4 : (n <= lanes * 17 / 32 ? 3 : 0);
 }
 
 template <int kP, bool kCount, bool kLeaves, bool kGroup>
@@ -1901,7 +1914,7 @@ static cudaError_t launch_tiled_t(cudaStream_t st, const TraceArgs &a, const Til
 template <int kP>
 static cudaError_t launch_tiled_p(cudaStream_t st, const TraceArgs &a0, const TiledArgs &ta, int n_sm) {
   TraceArgs a = a0;
-  a.group_log2 = group_log2<kP>(a.lineage_end - a.lineage_begin, n_sm);
+  a.group_log2 = group_log2<kP>(a.lineage_end - a.lineage_begin, n_sm, a.blocks_per_sm, true);
   if (a.leaf_size > 1)
     return a.count_work ? launch_tiled_t<kP, true, true, false>(st, a, ta, n_sm)
                         : launch_tiled_t<kP, false, true, false>(st, a, ta, n_sm);
@@ -2017,7 +2030,7 @@ static cudaError_t launch_trace_t(cudaStream_t st, const TraceArgs &a, int n_sm)
 template <int kP, bool kBatch>
 static cudaError_t launch_trace_p(cudaStream_t st, const TraceArgs &a0, int n_sm) {
   TraceArgs a = a0;
-  a.group_log2 = group_log2<kP>(a.lineage_end - a.lineage_begin, n_sm);
+  a.group_log2 = group_log2<kP>(a.lineage_end - a.lineage_begin, n_sm, a.blocks_per_sm, false);
   if (a.leaf_size > 1)
     return a.count_work ? launch_trace_t<kP, true, kBatch, true, false>(st, a, n_sm)
                         : launch_trace_t<kP, false, kBatch, true, false>(st, a, n_sm);

@@ -40,3 +40,9 @@ def test_reserved_lineages(city, tiles, sources, beams_per_warp):
 @pytest.mark.parametrize("sources,queue_depth", [(1, 32), (1, 1024), (2, 256), (8, 32), (8, 256), (8, 4096)])
 def test_shallow_queues(city, sources, queue_depth):
     check(city, sources, tiles_x=4, tiles_y=4, queue_depth=queue_depth)
+
+
+@pytest.mark.parametrize("tiles", [1, 4])
+@pytest.mark.parametrize("sources,blocks_per_sm", [(1, 1), (2, 1), (2, 2), (8, 1), (8, 2), (8, 4)])
+def test_fewer_blocks(city, tiles, sources, blocks_per_sm):
+    check(city, sources, tiles_x=tiles, tiles_y=tiles, blocks_per_sm=blocks_per_sm)
