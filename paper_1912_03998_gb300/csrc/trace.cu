@@ -1885,8 +1885,8 @@ static int group_log2(int64_t n, int n_sm, int blocks_per_sm, bool split) {
     const int64_t lanes = sm_lanes * blocks;
     return n <= lanes / 16 ? 4 : (n <= lanes * 3 / 8 ? 3 : 0);
   }
-  const int64_t lanes = sm_lanes * (blocks < 5 ? blocks : 5);
-  return n <= lanes * 3 / 32 ? 4 : (n <= lanes * 17 / 32 ? 3 : 0);
+  if (blocks < 5) return n <= sm_lanes * blocks * 3 / 32 ? 4 : (n <= sm_lanes * blocks * 17 / 32 ? 3 : 0);
+  return n <= sm_lanes * 7 / 16 ? 4 : (n <= sm_lanes * 7 * 3 / 8 ? 3 : 0);
 }
 
 template <int kP, bool kCount, bool kLeaves, bool kGroup>
