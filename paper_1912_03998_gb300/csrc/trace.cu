@@ -136,25 +136,47 @@ __global__ void k_beam_table(int level, int64_t n_beams, float *table) {
 // formed each lineage's beam in the trace kernel: some thousand float64
 // operations for the few lanes of a service phase that start a lineage, which
 // cost as much of the float64 pipe as everything else together (FP64, 24
-// district sources: trace kernel 3.23 -> 2.31 ms).
-__global__ void k_beam_table64(int level, int64_t n_beams, double *table) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n_beams) return;
-  double3 d0, d1, d2;
-  beam_dirs<double>(level, i, d0, d1, d2);
+// district sources: trace kernel 3.23 -> 2.31 ms).  From kBeamFaces on a thread
+// forms the four beams of one face of the level above, whose descent they
+// share: a call without allocation makes the table anew each time, and a beam a
+// thread took longer at level 6 than the trace saves by it (MIXED64, one source
+// in the 8 x 8-block city: 652 -> 602 us a call, 628 without a table).  Below,
+// the table is a chain of latencies, which four beams a thread lengthen (level
+// 4: 209 -> 217 us).
+constexpr int kBeamFaces = 5;
+__device__ __forceinline__ void put_beam64(double *o, double3 d0, double3 d1, double3 d2) {
   const double3 v[4] = {cross_exact(d0, d1), cross_exact(d1, d2), cross_exact(d2, d0), normalize3((d0 + d1) + d2)};
-  double *o = table + 12 * i;
+#pragma unroll
   for (int k = 0; k < 4; k++) {
     o[3 * k] = v[k].x;
     o[3 * k + 1] = v[k].y;
     o[3 * k + 2] = v[k].z;
   }
 }
+__global__ void k_beam_table64(int level, int64_t n_threads, double *table) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n_threads) return;
+  double3 a, b, c;
+  beam_dirs<double>(level < kBeamFaces ? level : level - 1, i, a, b, c);
+  if (level < kBeamFaces) {
+    put_beam64(table + 12 * i, a, b, c);
+    return;
+  }
+  const double3 ab = normalize3(a + b), bc = normalize3(b + c), ca = normalize3(c + a);
+  double *const o = table + 48 * i;
+  put_beam64(o, a, ab, ca);
+  put_beam64(o + 12, ab, b, bc);
+  put_beam64(o + 24, ca, bc, c);
+  put_beam64(o + 36, ab, bc, ca);
+}
 
 cudaError_t launch_beam_table(cudaStream_t st, int prec, int level, float *table) {
   int64_t n = (int64_t)20 << (2 * level);
   if (prec == kPMixed) k_beam_table<<<(int)((n + 127) / 128), 128, 0, st>>>(level, n, table);
-  else k_beam_table64<<<(int)((n + 127) / 128), 128, 0, st>>>(level, n, (double *)table);
+  else {
+    const int64_t threads = level < kBeamFaces ? n : n / 4;
+    k_beam_table64<<<(int)((threads + 127) / 128), 128, 0, st>>>(level, threads, (double *)table);
+  }
   note_launches(1);
   return cudaGetLastError();
 }

@@ -217,3 +217,15 @@ def test_microphones_by_a_triangle_of_many_km(tracer, oracle_mod, name):
         assert (g["cnt"] == r["cnt"]).all(), (seed, int((g["cnt"] != r["cnt"]).sum()))
         np.testing.assert_allclose(g["I"], r["I"], rtol=2e-6)
     assert found >= 3
+
+
+@pytest.mark.parametrize("level", [4, 5, 6])
+def test_float64_beams_on_both_sides_of_the_table_rule(tracer, oracle_mod, level):
+    """Free field: a microphone far from every edge lies in one beam, so a beam
+    formed for the wrong face shows as a missing or doubled count."""
+    w = synth.free_field(level=level, n_mics=4096)
+    for name in ("fp64", "mixed64"):
+        g = gpu_run(tracer, w, precision=prec(name))
+        r = oracle_mod.trace_workload(w)
+        assert (g["cnt"] == r["cnt"]).all()
+        np.testing.assert_allclose(g["I"], r["I"], rtol=2e-6)
