@@ -132,6 +132,7 @@ struct DevScene {
   float lo[3], hi[3];    // scene box
 };
 
+constexpr int kMaxLayers = 64;
 // Microphone bin grid over the microphones' box: nx x ny cells in xy and nz
 // layers in z (one layer for microphones at one height; several for a
 // volumetric set), cell (layer, row, column) = (iz * ny + iy) * nx + ix.
@@ -142,6 +143,10 @@ struct MicGrid {
   int n_mics;
   int nz;
   float z0, dz, inv_dz, pad;
+  // for the scatter over several layers: the layers that hold microphones, and
+  // how many (segment, layer) items a warp takes at most, as a power of two
+  int n_lay, take_log2;
+  unsigned char lay[kMaxLayers];
 };
 
 // One beam segment handed from the trace kernel to the scatter kernel, 192 B.

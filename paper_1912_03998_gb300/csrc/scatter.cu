@@ -262,7 +262,19 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   // segment, which for a long beam over the roofs hold tens of thousands of
   // candidates (13.75 M microphones, 8 sources: 40 % of the chip's time went
   // by waiting for such warps; 10.1 -> 5.9 ms, 40 sources 29.9 -> 24.6 ms).
-  const int n_layers = a.max_nz > 1 ? a.max_nz : 1;
+  // Only layers that hold microphones count, and fewer items are taken where the
+  // microphones crowd (k_mic_layers).
+  int n_layers = 1, most_log2 = 5;
+  if (a.max_nz > 1) {
+    if (kBatch) {
+      n_layers = a.max_nz;
+      for (int v = lane; v < a.n_views; v += 32) most_log2 = min(most_log2, a.views[v].grid->take_log2);
+      most_log2 = (int)__reduce_min_sync(0xffffffffu, (unsigned)most_log2);
+    } else {
+      n_layers = a.v.grid->n_lay;
+      most_log2 = a.v.grid->take_log2;
+    }
+  }
   const long long n_items = n_layers > 1 ? (n_seg + 31) / 32 * 32 * n_layers : n_seg;
   unsigned long long n_cand = 0, n_contrib = 0;
   // FP64: candidates that wait for their float64 test, (microphone, segment),
@@ -283,7 +295,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   // us).  The
   // next take is under way while a warp works.
   auto share = [&](long long left) {
-    int lg = 5;
+    int lg = most_log2;
     while (lg > 0 && left < n_warps << lg) lg--;
     return lg;
   };
@@ -321,6 +333,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
       const MicGrid &g = *(kBatch ? a.views[vi] : a.v).grid;
       // the footprint is clipped in the lane's own columns: the polygon rows
       // and, as scratch, the rows of the segment fields written below
+      if (a.max_nz > 1) layer = layer < g.n_lay ? (int)g.lay[layer] : g.nz;
       const int pn = layer < g.nz ? seg_footprint(sl, g, layer, PolyCol{&F[F_PX][lane], &F[F_PY][lane]},
                                                   PolyCol{&F[F_QX][lane], &F[F_QY][lane]})
                                   : 0;

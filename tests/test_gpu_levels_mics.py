@@ -86,3 +86,45 @@ def test_levels_are_rounded_once():
         err = np.array([abs(float(Decimal(float(y)) - r)) for y, r in zip(L.ravel(), ref)])
     tol = 0.5 * np.spacing(np.abs(np.array([float(r) for r in ref]))) + 1e-16
     assert (err <= tol).all(), (err / tol).max()
+
+
+@pytest.mark.parametrize("precision", [btrace.BT_PREC_MIXED, btrace.BT_PREC_FP64])
+@pytest.mark.parametrize("kind", ["planes", "clusters", "one off", "top and bottom", "column"])
+def test_layers_without_microphones(kind, precision):
+    """Volumes whose microphones fill few of the grid's layers or few of its
+    cells, alone and in a batch beside a planar set: free field, every
+    microphone once."""
+    rng = np.random.default_rng(len(kind))
+    n = 40000
+    m = rng.uniform(-80.0, 80.0, (n, 3))
+    if kind == "planes":
+        m[:, 2] = rng.choice([-3.0, 35.0], n)
+    if kind == "clusters":
+        m = rng.uniform(-60.0, 60.0, (7, 3))[rng.integers(0, 7, n)] + rng.uniform(0.0, 1.0, (n, 3))
+    if kind == "one off":
+        m[:, 2] = 1.5
+        m[n // 2, 2] = 70.0
+    if kind == "top and bottom":
+        m[:, 2] = np.where(rng.random(n) < 0.5, -40.0, 40.0) + rng.uniform(0.0, 0.1, n)
+    if kind == "column":
+        m[:, :2] = 20.0 + rng.uniform(0.0, 0.1, (n, 2))
+    w = synth.free_field(level=3).with_mics(m.astype(np.float32))
+    flat = synth.free_field(level=3)
+
+    def check(sid, mics, w):
+        I, cnt = np.empty((len(mics), 8)), np.empty(len(mics), np.int32)
+        btrace.bt_read_levels(t.ctx, sid, None, I, cnt)
+        assert (cnt == 1).all()
+        d2 = ((mics.astype(np.float64) - w.src[0].astype(np.float64)) ** 2).sum(1)
+        np.testing.assert_allclose(I, w.power[0].astype(np.float64)[None] / (4.0 * np.pi * d2[:, None]), rtol=1e-6)
+
+    with btrace.Tracer(0) as t:
+        sids = [t.load(w), t.load(flat)]
+        p = t.params(1, precision=precision)
+        btrace.bt_trace(t.ctx, sids[0], p)
+        check(sids[0], w.mics, w)
+        b = btrace.bt_batch_create(t.ctx, sids, [p, p])
+        btrace.bt_batch_run(t.ctx, b)
+        check(sids[0], w.mics, w)
+        check(sids[1], flat.mics, flat)
+        btrace.bt_batch_destroy(b)
