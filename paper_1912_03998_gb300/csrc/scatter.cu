@@ -292,8 +292,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   // which a warp tests 32 at a time -- so with fixed shares a launch lasted as
   // long as its fullest warp (eight uneven cities, 4.4 M segments: batch call
   // 5.0 -> 4.3 ms; 17,700 segments of 28 candidates each on average: 617 -> 121
-  // us).  The
-  // next take is under way while a warp works.
+  // us).  The next take is under way while a warp works.
   auto share = [&](long long left) {
     int lg = most_log2;
     while (lg > 0 && left < n_warps << lg) lg--;
@@ -487,56 +486,56 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
             near = near && dot3(ns, v) - F[F_NS + 3][s] >= -side && dot3(ne, v) - F[F_NE + 3][s] >= -side;
             if (near) entry = make_int2(mi, __float_as_int(F[F_SI][s]));
           } else {
-          // cone planes: float32; within the rounding band of a plane the
-          // test is redone with float pairs
-          const float band_v = 2e-6f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z));
-          bool in = true;
+            // cone planes: float32; within the rounding band of a plane the
+            // test is redone with float pairs
+            const float band_v = 2e-6f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z));
+            bool in = true;
 #pragma unroll
-          for (int j = 0; j < 3; j++) {
-            float3 nj = make_float3(F[F_N0 + 3 * j][s], F[F_N0 + 3 * j + 1][s], F[F_N0 + 3 * j + 2][s]);
-            float e = dot3(nj, v);
-            if (fabsf(e) <= band_v * (fabsf(nj.x) + fabsf(nj.y) + fabsf(nj.z))) {
-              df3 nd = df3{df{nj.x, __ldg(&rec->nlo[3 * j])}, df{nj.y, __ldg(&rec->nlo[3 * j + 1])},
-                           df{nj.z, __ldg(&rec->nlo[3 * j + 2])}};
-              df ed = df3_dot(nd, rel_df(F, s, m));
-              e = ed.hi + ed.lo;
+            for (int j = 0; j < 3; j++) {
+              float3 nj = make_float3(F[F_N0 + 3 * j][s], F[F_N0 + 3 * j + 1][s], F[F_N0 + 3 * j + 2][s]);
+              float e = dot3(nj, v);
+              if (fabsf(e) <= band_v * (fabsf(nj.x) + fabsf(nj.y) + fabsf(nj.z))) {
+                df3 nd = df3{df{nj.x, __ldg(&rec->nlo[3 * j])}, df{nj.y, __ldg(&rec->nlo[3 * j + 1])},
+                             df{nj.z, __ldg(&rec->nlo[3 * j + 2])}};
+                df ed = df3_dot(nd, rel_df(F, s, m));
+                e = ed.hi + ed.lo;
+              }
+              in = in && e >= 0.0f;
             }
-            in = in && e >= 0.0f;
-          }
-          if (in) {
-            // start/end planes: float32 relative to the apex; within the
-            // rounding band the test is redone with float pairs against the
-            // triangle's own plane, the form the definition uses
-            float3 ns = make_float3(F[F_NS][s], F[F_NS + 1][s], F[F_NS + 2][s]);
-            float3 ne = make_float3(F[F_NE][s], F[F_NE + 1][s], F[F_NE + 2][s]);
-            float band = 1e-4f + 1e-6f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z));
-            float fs = dot3(ns, v) - F[F_NS + 3][s], fe = dot3(ne, v) - F[F_NE + 3][s];
-            if (fabsf(fs) <= band || fabsf(fe) <= band) {
-              const SceneView &V = kBatch ? a.views[__float_as_int(F[F_VI][s])] : a.v;
-              int s_slot = __float_as_int(__ldg(&rec->n0.w)), e_slot = __float_as_int(__ldg(&rec->n1.w));
-              if (fabsf(fs) <= band && s_slot >= 0) fs = plane_side_df(V, s_slot, ns, m);
-              if (fabsf(fe) <= band && e_slot >= 0) fe = plane_side_df(V, e_slot, ne, m);
+            if (in) {
+              // start/end planes: float32 relative to the apex; within the
+              // rounding band the test is redone with float pairs against the
+              // triangle's own plane, the form the definition uses
+              float3 ns = make_float3(F[F_NS][s], F[F_NS + 1][s], F[F_NS + 2][s]);
+              float3 ne = make_float3(F[F_NE][s], F[F_NE + 1][s], F[F_NE + 2][s]);
+              float band = 1e-4f + 1e-6f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z));
+              float fs = dot3(ns, v) - F[F_NS + 3][s], fe = dot3(ne, v) - F[F_NE + 3][s];
+              if (fabsf(fs) <= band || fabsf(fe) <= band) {
+                const SceneView &V = kBatch ? a.views[__float_as_int(F[F_VI][s])] : a.v;
+                int s_slot = __float_as_int(__ldg(&rec->n0.w)), e_slot = __float_as_int(__ldg(&rec->n1.w));
+                if (fabsf(fs) <= band && s_slot >= 0) fs = plane_side_df(V, s_slot, ns, m);
+                if (fabsf(fe) <= band && e_slot >= 0) fe = plane_side_df(V, e_slot, ne, m);
+              }
+              in = fs > 0.0f && fe >= 0.0f;
             }
-            in = fs > 0.0f && fe >= 0.0f;
-          }
-          float d2 = dot3(v, v);
-          if (in && d2 > 1e-18f) {
-            float gf = 1.0f / (4.0f * 3.14159265358979f * d2);
-            float dist = has_alpha ? sqrtf(d2) : 0.0f;
-            double *e = energy + (size_t)mi * kMaxBands;
-            if (has_alpha) {
-              const float *alpha = (kBatch ? a.views[__float_as_int(F[F_VI][s])] : a.v).alpha_log2;
+            float d2 = dot3(v, v);
+            if (in && d2 > 1e-18f) {
+              float gf = 1.0f / (4.0f * 3.14159265358979f * d2);
+              float dist = has_alpha ? sqrtf(d2) : 0.0f;
+              double *e = energy + (size_t)mi * kMaxBands;
+              if (has_alpha) {
+                const float *alpha = (kBatch ? a.views[__float_as_int(F[F_VI][s])] : a.v).alpha_log2;
 #pragma unroll
-              for (int b = 0; b < kMaxBands; b++)
-                if (b < nb) atomicAdd(e + b, (double)(F[F_P + b][s] * gf * exp2f(alpha[b] * dist)));
-            } else {
+                for (int b = 0; b < kMaxBands; b++)
+                  if (b < nb) atomicAdd(e + b, (double)(F[F_P + b][s] * gf * exp2f(alpha[b] * dist)));
+              } else {
 #pragma unroll
-              for (int b = 0; b < kMaxBands; b++)
-                if (b < nb) atomicAdd(e + b, (double)(F[F_P + b][s] * gf));
+                for (int b = 0; b < kMaxBands; b++)
+                  if (b < nb) atomicAdd(e + b, (double)(F[F_P + b][s] * gf));
+              }
+              atomicAdd(&count[mi], 1);
+              n_contrib++;
             }
-            atomicAdd(&count[mi], 1);
-            n_contrib++;
-          }
           }
         }
         if (kF64) {

@@ -255,16 +255,6 @@ __device__ __forceinline__ bool pend_add(const RaySrc &rs, int entry) {
   return true;
 }
 
-// Closest accepted hit of the ray in the BVH; ties in distance go to the
-// lowest original triangle id.  In the deferring variants `rs` gives the
-// float-pair or float64 ray that the float32 ray `r` rounds, read only on the
-// rare float64 paths.
-// Returns the leaf slot or -1.
-
-// Candidate triangle `slot` against the best hit so far (ties in distance go
-// to the lowest original triangle id).  With MIXED/FP64, `rs` gives the
-// float-pair or float64 ray that the float32 ray `r` rounds, read only on the
-// float64 paths.  Hits beyond `tlim` are ignored.
 // An event count of a warp, in shared memory: every lane that passes an
 // increment adds one, the lanes that execute it together with one atomic.
 struct WarpCount {
@@ -693,16 +683,16 @@ __device__ __forceinline__ void search_phase(const DevScene &sc, bool lane_tris,
 // ------------------------------------------------------- groups of lanes
 // Small launches: fewer lineages than the chip has lanes.  Their time is the
 // latency of the longest lineage, one dependent node fetch after the other, so
-// a group of G = 8, 16 or 32 lanes works on one lineage: a step takes the top
+// a group of G = 8 or 16 lanes works on one lineage: a step takes the top
 // G / 4 nodes of the group's stack at once, four lanes to a node and one child
 // box to a lane.
-constexpr int kGroupMin = 8;                               // lanes
+constexpr int kGroupMin = 8, kGroupMax = 16;               // lanes
 constexpr int kGroupCols = kTraceThreads / kGroupMin;      // groups in a block
 // A group takes several nodes a step only while its stack is shallow, so that
 // taking one at a time from there on (at most three more entries per level of
 // the binary hierarchy, kStackDepth in all) still fits.
 constexpr int kGroupShallow = 40;
-constexpr int kGroupDepth = kGroupShallow + 3 * (32 / 4) + kStackDepth;
+constexpr int kGroupDepth = kGroupShallow + 3 * (kGroupMax / 4) + kStackDepth;
 constexpr int kGroupPairTest = 8;
 struct GroupStack {
   int node[kGroupCols][kGroupDepth];
@@ -721,7 +711,7 @@ __device__ __forceinline__ void search_groups(const DevScene &sc, bool lane_tris
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = (int)lane_id(), G = 1 << lg;
   const int leader = lane & ~(G - 1), sub = lane & 3, q = (lane & (G - 1)) >> 2;
-  const unsigned group = G == 32 ? kAll : (1u << G) - 1u;
+  const unsigned group = (1u << G) - 1u;
   const Tri *const tris = sc.tris;
   const float3 inv = r.inv, oi = origin_scaled(r);
   const char *const nodes = (const char *)sc.nodes + 4 * sub;
@@ -1878,15 +1868,19 @@ __global__ void __launch_bounds__(kTraceThreads, kP == kPF32 || kP == kPMixed ? 
 // Lanes that work on one lineage, as a power of two, for a launch of n
 // lineages: 16 or 8 while the chip's lanes (seven blocks per SM) are enough to
 // give every lineage some, which its chain of dependent fetches needs more than
-// the launch needs throughput.  Measured (trace kernel, us, 1 / 8 / 16 / 32
-// lanes per lineage; district and an 8 x 8-block city, order 4, MIXED):
-//   lineages   5,120  159/83/73/77 and 139/74/66/79
-//             10,240  245/123/107/132 and 146/79/86/131
-//             40,960  317/214/277/445 and 166/159/225/368
-//             61,440  328/299/406/674 and 202/212/309/511
-// split 4 x 4: 5,120 385/333/336/352, 40,960 968/634/767/966.  Not for the
-// float64 chain, which leaves too much to one lane of a group (FP64 at 10,240
-// lineages 344/245/332/541 and 225/249/374/623).
+// the launch needs throughput.  Measured (trace kernel, us, 1 / 8 / 16 lanes per
+// lineage; district and an 8 x 8-block city, order 4, MIXED):
+//   lineages   5,120  170/77/65 and 134/63/59
+//             10,240  168/79/75 and 139/69/77
+//             40,960  280/180/231 and 155/141/201
+//             61,440  301/216/292 and 191/188/280
+//   split 4 x 4  5,120  350/165/223 and 393/149/210
+//               40,960  688/571/671 and 491/542/673
+// (32 lanes were slower than 16 everywhere.)  There are no group kernels for the float64
+// chain and for FP32 split: on the city 8 lanes would pay below some 10,000 and
+// 30,000 lineages (5,120, 10,240, 40,960: FP64 200/128/163, 202/182/258,
+// 244/489/778; MIXED64 151/92/124, 157/114/174, 176/303/535; FP32 split
+// 323/129/180, 387/215/325, 426/444/525), which is left to be taken up.
 // A warp of groups holds 32 >> log2 lineages, so it reserves that share of
 // beams_per_warp: with all of it a warp went through its reservation two at a
 // time while others had none (8 x 8-block city, 5,120 lineages, 256 a warp: 4.79
@@ -1941,8 +1935,6 @@ static cudaError_t launch_tiled_p(cudaStream_t st, const TraceArgs &a0, const Ti
     return a.count_work ? launch_tiled_t<kP, true, true, false>(st, a, ta, n_sm)
                         : launch_tiled_t<kP, false, true, false>(st, a, ta, n_sm);
   if (a.count_work) return launch_tiled_t<kP, true, false, false>(st, a, ta, n_sm);
-  // (FP32's chain rounds by each kernel's own contractions, so it keeps to the
-  // kernel that larger launches run)
   if constexpr (kP == kPMixed)
     if (a.group_log2 > 0) {
       a.beams_per_warp >>= a.group_log2;
