@@ -835,20 +835,20 @@ __global__ void k_mic_keys(const float *pos, int64_t n, const MicGrid *g, uint32
 }
 
 // What the scatter over several layers wants to know of them (k_scatter).
-// Layers without microphones are left out: two planes 38 m apart hold all of a
-// grid's 27 layers in two, and clipping segments against the others took a
-// third of the scatter (1 M microphones, 64 sources: 7.8 -> 4.5 ms).  Where
+// Layers without microphones are left out: two planes 38 m apart fill two of a
+// grid's 17 layers, and clipping segments against the others took 40 % of the
+// scatter (1 M microphones, 64 sources: 7.8 -> 4.6 ms).  Where
 // the microphones crowd into few cells a take is four items instead of 32: one
 // layer of 32 segments then holds a million candidates and the launch waits for
 // few warps (1 M microphones in 27 cubic metres, 16 sources: 17.8 -> 5.0 ms;
 // takes of four would cost a uniform volume 2.5 times its time).  Measured by
 // the population of a microphone's cell, mean over a sample: about 5 in a
 // uniform volume, 10 to 100 on planes and facades, thousands in such clusters.
-constexpr int kCrowded = 512, kLayerThreads = 1024, kLayerSample = 4;
-__global__ void __launch_bounds__(kLayerThreads) k_mic_layers(const uint2 *place, int64_t n, const int *cell_start,
-                                                              MicGrid *g) {
+// One block of k_mic_place does it (a launch of its own took 8 us of 94).
+constexpr int kCrowded = 512, kPlaceThreads = 256, kLayerSample = 16;
+__device__ __forceinline__ void mic_layers(const uint2 *place, int64_t n, const int *cell_start, MicGrid *g) {
   const int t = threadIdx.x, lane = t & 31, per_layer = g->nx * g->ny;
-  __shared__ float part[kLayerThreads / 32];
+  __shared__ float part[kPlaceThreads / 32];
   __shared__ int first;
   const int l = t < kMaxLayers && t < g->nz ? t : -1;
   const bool holds = l >= 0 && cell_start[(l + 1) * per_layer] > cell_start[l * per_layer];
@@ -858,20 +858,23 @@ __global__ void __launch_bounds__(kLayerThreads) k_mic_layers(const uint2 *place
   if (holds) g->lay[(t >= 32 ? first : 0) + __popc(b & ((1u << lane) - 1u))] = (unsigned char)l;
   if (t == 32) g->n_lay = first + __popc(b);
   float sum = 0.0f;
+#pragma unroll 4
   for (int q = 0; q < kLayerSample; q++) {
-    const uint32_t c = place[(int64_t)(t * kLayerSample + q) * n / (kLayerThreads * kLayerSample)].x;
+    const uint32_t c = place[(int64_t)(q * kPlaceThreads + t) * n / (kPlaceThreads * kLayerSample)].x;
     sum += (float)(cell_start[c + 1] - cell_start[c]);
   }
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) part[t >> 5] = sum;
   __syncthreads();
   if (t == 0) {
-    for (int w = 1; w < kLayerThreads / 32; w++) sum += part[w];
-    g->take_log2 = sum > (float)kCrowded * (kLayerThreads * kLayerSample) ? 2 : 5;
+    for (int w = 1; w < kPlaceThreads / 32; w++) sum += part[w];
+    g->take_log2 = sum > (float)kCrowded * (kPlaceThreads * kLayerSample) ? 2 : 5;
   }
 }
 
-__global__ void k_mic_place(const float *pos, int64_t n, const int *cell_start, const uint2 *place, float4 *sorted) {
+__global__ void __launch_bounds__(kPlaceThreads) k_mic_place(const float *pos, int64_t n, const int *cell_start,
+                                                             const uint2 *place, float4 *sorted, MicGrid *g) {
+  if (g && blockIdx.x == 0) mic_layers(place, n, cell_start, g);
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint2 p = place[i];
@@ -903,12 +906,11 @@ cudaError_t build_mics(cudaStream_t st, const float *d_pos, int64_t n_m, int nx,
   // counts, and zero behind them: the scan leaves the starts and the total
   cudaError_t e = cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (n_cells + 1), st);
   if (e != cudaSuccess || n_m == 0) return e;
-  const int threads = 256, blocks = (int)((n_m + threads - 1) / threads);
+  const int threads = kPlaceThreads, blocks = (int)((n_m + threads - 1) / threads);
   k_mic_keys<<<blocks, threads, 0, st>>>(d_pos, n_m, d_grid, (uint32_t *)d_cell_start, place);
   k_scan_excl<<<1, 1024, 0, st>>>((uint32_t *)d_cell_start, n_cells + 1);
-  k_mic_place<<<blocks, threads, 0, st>>>(d_pos, n_m, d_cell_start, place, d_sorted);
-  if (nz > 1) k_mic_layers<<<1, kLayerThreads, 0, st>>>(place, n_m, d_cell_start, d_grid);
-  note_launches(nz > 1 ? 4 : 3);
+  k_mic_place<<<blocks, threads, 0, st>>>(d_pos, n_m, d_cell_start, place, d_sorted, nz > 1 ? d_grid : nullptr);
+  note_launches(3);
   return cudaGetLastError();
 }
 

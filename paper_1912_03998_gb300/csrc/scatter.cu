@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(32 * kScatterWarps) k_scatter(ScatterArgs a) {
   // candidates (13.75 M microphones, 8 sources: 40 % of the chip's time went
   // by waiting for such warps; 10.1 -> 5.9 ms, 40 sources 29.9 -> 24.6 ms).
   // Only layers that hold microphones count, and fewer items are taken where the
-  // microphones crowd (k_mic_layers).
+  // microphones crowd (mic_layers).
   int n_layers = 1, most_log2 = 5;
   if (a.max_nz > 1) {
     if (kBatch) {
