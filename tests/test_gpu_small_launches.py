@@ -72,3 +72,35 @@ def test_groups_in_a_batch():
         for (I0, c0), (I1, c1) in zip(got[:3], got[3:]):
             assert (c0 == c1).all()
             np.testing.assert_allclose(I0, I1, rtol=1e-9, atol=0.0)
+
+
+def test_groups_few_triangles_split():
+    """Sub-domains with hierarchies of one leaf, of a few, and of none."""
+    with btrace.Tracer(0) as t:
+        for w in (synth.boxes(1, level=3), synth.boxes(4, level=3), synth.ground_only(level=3), synth.single_wall(level=3)):
+            both(t, t.load(w), len(w.mics), 8, w.max_order, tiles_x=3, tiles_y=4)
+        w = synth.ground_only(level=3)
+        w.scene.tris, w.scene.mat = w.scene.tris[:1], w.scene.mat[:1]
+        both(t, t.load(w), len(w.mics), 8, w.max_order, tiles_x=5, tiles_y=2)
+
+
+@pytest.mark.parametrize("precision", [btrace.BT_PREC_FP32, btrace.BT_PREC_MIXED])
+def test_chunks_on_both_sides_of_the_rule(precision):
+    """A lineage rounds alike whatever the size of its launch: 163,840 lineages in
+    one launch on single lanes, in chunks of 60,000 with the rest on groups of
+    eight, in chunks of 45,000 on those and of 7,000 on groups of sixteen."""
+    w = synth.tiny_city(seed=6, level=5, max_order=5, n_grid=40, n_sources=8)
+    with btrace.Tracer(0) as t:
+        sid = t.load(w)
+        out = []
+        for chunk in (0, 60000, 45000, 7000):
+            btrace.bt_trace(t.ctx, sid, t.params(w.max_order, precision=precision, chunk_beams=chunk))
+            I, cnt = np.empty((len(w.mics), 8)), np.empty(len(w.mics), np.int32)
+            st = btrace.bt_read_levels(t.ctx, sid, None, I, cnt)
+            out.append((I, cnt, st))
+        for I, cnt, st in out[1:]:
+            for k in ("segments", "hits", "escapes", "emitted", "contributions"):
+                assert st[k] == out[0][2][k], k
+            assert (cnt == out[0][1]).all()
+            # (float32 contributions in float64 sums: only their order differs)
+            np.testing.assert_allclose(I, out[0][0], rtol=1e-12, atol=0.0)
